@@ -410,6 +410,11 @@ struct prism_plan {
     float2 *twr_f = nullptr, *twr_i = nullptr, *twc_f = nullptr, *twc_i = nullptr, *tww_f = nullptr, *tww_fy = nullptr;
     int *beam_mn = nullptr;
     double *beam_q = nullptr;  // qx[B] then qy[B]
+    int *m_off = nullptr, *m_beam = nullptr;  // the beams by m (ScanArgs::m_off)
+    double *m_qx = nullptr;
+    int rows_m = 0, rows_maxn = 0;
+    float2 *rows_w = nullptr;  // sums over n of the raster-row scan
+    size_t rows_cap = 0;
     // grown on demand
     double *pos = nullptr;
     size_t pos_cap = 0;
@@ -419,6 +424,7 @@ struct prism_plan {
     size_t bin_t_off = 0;      // element offset of the by-rank table in bin_buf
     size_t bin_16_off = 0;     // element offset of the 16-bit lists in bin_buf (a multiple of 4)
     size_t bin_n = 0;          // entries of the lists
+    size_t fold_off = 0, fold_n = 0;  // the folded quadrant's lists: element offset (a multiple of 4), 16-bit entries
     float *out_stage = nullptr;
     size_t out_cap = 0;
     float *v_stage = nullptr;
@@ -690,6 +696,21 @@ extern "C" int prism_plan_create(const prism_grid *grid, size_t hbm_budget_bytes
     if ((rc = A.upload(&P->tww_fy, tww_fy))) return bail(rc);
     if ((rc = A.upload(&P->beam_mn, mn))) return bail(rc);
     if ((rc = A.upload(&P->beam_q, q))) return bail(rc);
+    // the beams by m = -M ... M (the set is symmetric in m), n ascending
+    std::vector<int> m_off, m_beam;
+    std::vector<double> m_qx;
+    for (int b = 0; b < P->nbeams; ++b) P->rows_m = std::max(P->rows_m, P->bm[b]);
+    for (int m = -P->rows_m; m <= P->rows_m; ++m) {
+        m_off.push_back((int)m_beam.size());
+        for (int b = 0; b < P->nbeams; ++b)
+            if (P->bm[b] == m) m_beam.push_back(b);
+        P->rows_maxn = std::max(P->rows_maxn, (int)m_beam.size() - m_off.back());
+        if (m >= 0) m_qx.push_back((double)(m * g.f) / g.cell_x);
+    }
+    m_off.push_back((int)m_beam.size());
+    if ((rc = A.upload(&P->m_off, m_off))) return bail(rc);
+    if ((rc = A.upload(&P->m_beam, m_beam))) return bail(rc);
+    if ((rc = A.upload(&P->m_qx, m_qx))) return bail(rc);
     if ((rc = A.alloc((void **)&P->base, (size_t)P->nbeams * sizeof(float2)))) return bail(rc);
     // the uploads above read host vectors that die with this scope
     cudaError_t e = cudaStreamSynchronize(P->stream);
@@ -935,6 +956,57 @@ extern "C" int prism_build_smatrix_host(prism_plan *P, const float *V_host) {
 }
 
 // ------------------------------------------------------------------ scan
+// Whether the scan goes by raster rows (scan_rows.cuh), and its geometry: FP32 S-matrix, every row of
+// the raster on one y, rows of 3 probes or more, and few enough columns under the rows' windows.  A row's
+// sums cost one product per beam and column reached, then each probe one per distinct m and window pixel;
+// in blocks (scan_gemm.cuh) each probe costs one per beam and window pixel.  Measured over windows of 32
+// to 128 pixels, 49 to 529 beams, steps of 0.1 to 2 A and rasters of 2 x 2 to 64 x 64: 1.2 to 6.6 times
+// the speed of the blocks wherever the test below lets rows of 3 or more through, 0.84 to 1.06 times for
+// tall rasters of rows of 2.  Sets a.rows_lp > 0, the columns and the rows held at once, or leaves
+// a.rows_lp = 0.
+static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) {
+    if (P->prec != PRISM_PRECISION_FP32 || sc->px < 3 || sc->py < 1) return;
+    double xmin = sc->x0[0], xmax = sc->x0[0];
+    for (int r = 0; r < sc->py; ++r) {
+        const double *x = sc->x0 + (size_t)r * sc->px, *y = sc->y0 + (size_t)r * sc->px;
+        for (int i = 0; i < sc->px; ++i) {
+            if (y[i] != y[0]) return;
+            xmin = std::min(xmin, x[i]);
+            xmax = std::max(xmax, x[i]);
+        }
+    }
+    // columns from the first window's to the last one's, to whole runs of 16 (positions reach 2^28 pixels)
+    const long long first = (long long)std::floor(xmin / a.px_s + 0.5) - P->nw / 2;
+    const long long last = (long long)std::floor(xmax / a.px_s + 0.5) - P->nw / 2 + P->nw;
+    const long long g0 = first & ~15LL;
+    const long long reach = (last - g0 + 15) & ~15LL;
+    const int cols = (int)std::min<long long>(reach, P->nxs);
+    const int planes = 2 * P->rows_m + 1;
+    if ((double)cols * P->nbeams + (double)sc->px * P->nw * planes > 0.75 * (double)sc->px * P->nw * P->nbeams) return;
+    // rows held at once: no more memory than the blocks' window scratch would take (32 windows per
+    // block of 4 x 4, two blocks per SM at most, twice over for split blocks), and 384 MB (1.53 ms for the
+    // 200 x 200 probes of the carbon cell, two launches each of 100 rows; 192 MB: 1.64 ms, 640 MB: 1.52)
+    const size_t row = (size_t)P->nwy * planes * cols * sizeof(float2);
+    const size_t blocks = ((size_t)sc->px + 3) / 4 * (((size_t)sc->py + 3) / 4);
+    const size_t most = std::min<size_t>(std::min<size_t>(blocks, 304) * 64 * P->nw * P->nwy * sizeof(float2), (size_t)384 << 20);
+    size_t chunk = std::min<size_t>(most / row, sc->py);
+    if (chunk == 0) return;
+    // in equal shares, to whole groups of 4
+    chunk = ((size_t)sc->py + (sc->py + chunk - 1) / chunk - 1) / ((sc->py + chunk - 1) / chunk);
+    if (chunk % 4 && chunk < (size_t)sc->py && (chunk + 3) / 4 * 4 * row <= most) chunk = (chunk + 3) / 4 * 4;
+    const int lp = scan_rows_lp(P->nw, P->nwy, P->rows_m, P->rows_maxn, a.n_fold16, sc->px, (int)chunk);
+    if (lp <= 0) return;
+    a.rows_lp = lp;
+    a.rows_m = P->rows_m;
+    a.rows_maxn = P->rows_maxn;
+    a.m_off = P->m_off;
+    a.m_beam = P->m_beam;
+    a.m_qx = P->m_qx;
+    a.rows_g0 = cols == P->nxs ? 0 : (int)(((g0 % P->nxs) + P->nxs) % P->nxs);
+    a.rows_cols = cols;
+    a.rows_chunk = (int)chunk;
+}
+
 static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_scan *sc, const prism_detector *det,
                         ScanArgs &a, bool need_built = true) {
     int rc;
@@ -996,6 +1068,22 @@ static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_sca
         const size_t w16 = i16.size() / 2;
         all.resize(all.size() + w16);
         std::memcpy(all.data() + P->bin_16_off, i16.data(), i16.size() * sizeof(uint16_t));
+        // the quadrant 0 <= kx <= nw_x/2, 0 <= ky <= nw_y/2 alone (a pixel's bin depends on |kx| and |ky|;
+        // index nw/2 is its own mirror), for the scans that fold the intensities onto it first
+        std::vector<uint16_t> fold(det->nbins + 1, 0);
+        for (int k = 0; k < det->nbins; ++k) {
+            for (int i = off[k]; i < off[k + 1]; ++i) {
+                const int ky = idx[i] / P->nw, kx = idx[i] - ky * P->nw;
+                if (kx <= P->nw / 2 && ky <= P->nwy / 2) fold.push_back((uint16_t)(ky * (P->nw / 2 + 1) + kx));
+            }
+            fold[k + 1] = (uint16_t)(fold.size() - (det->nbins + 1));
+        }
+        fold.resize((fold.size() + 7) / 8 * 8, 0);
+        while (all.size() % 4) all.push_back(0);
+        P->fold_off = all.size();
+        P->fold_n = fold.size();
+        all.resize(all.size() + fold.size() / 2);
+        std::memcpy(all.data() + P->fold_off, fold.data(), fold.size() * sizeof(uint16_t));
         if ((rc = grow(P->arena, (void **)&P->bin_buf, &P->bin_cap, all.size() * sizeof(int)))) return rc;
         CUDA_TRY(cudaMemcpyAsync(P->bin_buf, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, P->stream));
         P->det_nbins = det->nbins;
@@ -1034,7 +1122,10 @@ static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_sca
     a.scan_px = sc->px;
     a.scan_py = sc->py;
     a.err = P->dev_err;
+    a.fold16 = det ? reinterpret_cast<const uint16_t *>(P->bin_buf + P->fold_off) : nullptr;
+    a.n_fold16 = det ? (int)P->fold_n : 0;
     a.tw = P->tw64;
+    raster_rows(P, sc, a);
     return PRISM_OK;
 }
 
@@ -1053,7 +1144,7 @@ static int split_counters(prism_plan *P, ScanArgs &a, int grid) {
 
 // FP32 mode: the CUDA-core scan kernels; 16-bit mode: the tensor-core kernel (persistent grid, its
 // window scratch grown on demand)
-// FP32: the GEMM scan over 8 x 4 raster blocks when its shared memory fits (grid > 0), else the
+// FP32: the raster-row scan where it applies (raster_rows), the GEMM scan over 8 x 4 raster blocks when its shared memory fits (grid > 0), else the
 // grouped / per-probe kernels (grid 0); 16-bit: the tensor-core scan
 // the GEMM scan's contraction shape in use: the tuned or pinned one where it is compiled for the
 // plan's window, else the default
@@ -1068,6 +1159,14 @@ static int tc_shape(const prism_plan *P) {
 
 static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
     *grid = 0;
+    if (a.rows_lp > 0) {
+        const size_t wb = (size_t)a.rows_chunk * P->nwy * (2 * a.rows_m + 1) * a.rows_cols * sizeof(float2);
+        int rc = grow(P->arena, (void **)&P->rows_w, &P->rows_cap, wb);
+        if (rc) return rc;
+        a.rows_w = P->rows_w;
+        *grid = 1;
+        return PRISM_OK;
+    }
     if (P->prec == PRISM_PRECISION_FP32) {
         const int sh = gemm_shape(P);
         *grid = scan_gemm_grid(P->nw, P->nwy, sh, P->nbeams, a.scan_px, a.scan_py);
@@ -1089,6 +1188,11 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
 }
 
 static int scan_go(prism_plan *P, const ScanArgs &a, int grid) {
+    if (a.rows_lp > 0) {
+        const int rc = plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_rows(P->nw, P->nwy, a, P->stream); });
+        if (!rc) P->launches += 2 * ((a.scan_py + a.rows_chunk - 1) / a.rows_chunk) - 1;  // two kernels per chunk of rows
+        return rc;
+    }
     if (P->prec == PRISM_PRECISION_FP32)
         return plan_launch(P, PRISM_K_SCAN, [&] {
             return grid > 0 ? launch_scan_gemm(P->nw, P->nwy, gemm_shape(P), grid, a, P->stream)
@@ -1788,11 +1892,19 @@ extern "C" int prism_plan_autotune_scan(prism_plan *P, const prism_probe *probe,
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
-    int best = 0;
+    // a scan by raster rows has no contraction blocks: timed once, the same for every shape, and the
+    // plan's shape stays (position lists use it)
+    const bool rows = a.rows_lp > 0;
+    const int kept = P->scan_shape;
+    int best = rows ? kept : 0;
     double best_ms = -1.0;
     for (int v = 0; v < scan_gemm_shapes() && v < PRISM_TUNE_MAX_SHAPES && !rc; ++v) {
         if (!scan_gemm_shape_valid(P->nw, P->nwy, v)) continue;
-        P->scan_shape = v;
+        if (rows && best_ms >= 0) {
+            P->scan_ms[v] = best_ms;
+            continue;
+        }
+        if (!rows) P->scan_shape = v;
         int grid = 0;
         if ((rc = scan_setup(P, a, &grid))) break;
         if (grid <= 0) continue;  // this shape's coefficient block does not fit shared memory
@@ -1810,7 +1922,7 @@ extern "C" int prism_plan_autotune_scan(prism_plan *P, const prism_probe *probe,
         }
         P->scan_ms[v] = ms / 2.0;
         if (best_ms < 0 || ms / 2.0 < best_ms) {
-            best = v;
+            best = rows ? kept : v;
             best_ms = ms / 2.0;
         }
     }

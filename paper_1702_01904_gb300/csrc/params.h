@@ -120,6 +120,20 @@ struct ScanArgs {
     int *err;                  // device error word (a bounded wait that ran out sets bit 0)
     int kp;                    // K = 2 * roundup(B, 8)
     int scan_px, scan_py;      // probe raster, probe index = row * scan_px + col
+    // raster rows of one y each (scan_rows.cuh); rows_lp = 0: not such a scan
+    const int *m_off;          // [2 M + 2] CSR over m = -M ... M: the beams of m, n ascending
+    const int *m_beam;         // [B]
+    const double *m_qx;        // [M + 1] qx of the beams m = 0 ... M
+    int rows_m;                // M
+    int rows_maxn;             // beams of one m at most
+    float2 *rows_w;            // [rows_chunk][nw_y][2 M + 1][rows_cols] transformed sums over n
+    int rows_g0, rows_cols;    // columns held: rows_g0 ... rows_g0 + rows_cols - 1 (mod nx_s), multiples of 16
+    int rows_chunk;            // raster rows whose sums are held at once
+    int rows_lp;               // probes per CTA
+    int rows_0, rows_n;        // set per launch: first raster row, raster rows
+    const uint16_t *fold16;    // the bins over the quadrant 0 <= kx <= nw_x/2, 0 <= ky <= nw_y/2: CSR offsets
+                               // [nbins + 1], then the lists (ky * (nw_x/2 + 1) + kx); 16-byte aligned
+    int n_fold16;              // its entries, padded to 8 (0: no bins)
     Tw64 tw;
 };
 
@@ -181,6 +195,11 @@ cudaError_t launch_scan_gemm_tuned(int nwx, int nwy, int shape, int grid, const 
 // scan counters: completion counters of the split groups (int[grid]), the next work unit and the
 // CTAs done (int[2]); zeroed once, each launch leaves them zero
 size_t scan_gemm_cnt_bytes(int grid);
+// the raster-row scan (scan_rows.cuh): probes per CTA for rows of px probes
+// and so many 16-bit entries of bin lists (0: these windows, beams
+// or sizes are not for it), launch
+int scan_rows_lp(int nwx, int nwy, int m, int max_beams, int lists, int px, int rows);
+cudaError_t launch_scan_rows(int nwx, int nwy, const ScanArgs &a, cudaStream_t s);
 cudaError_t launch_shift(const ShiftArgs &a, cudaStream_t s);
 cudaError_t launch_bins(const BinArgs &a, cudaStream_t s);
 cudaError_t launch_tc_selftest(float *out, int *status, cudaStream_t s);

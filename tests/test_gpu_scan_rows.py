@@ -1,0 +1,105 @@
+"""The raster-row scan (rows of one y each) against the general scan of the same positions, on an S-matrix of
+random values, at the edges of its tiles: windows of every size and shape, rows of 3 probes and of more
+than one CTA's, steps below a pixel and wider than a window, rows that wrap, run backwards or shift, and
+beam sets of one m up to several chunks of pairs."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1702_01904_gb300 import prism as P  # noqa: E402
+from paper_1702_01904_gb300.runtime import PrismSimulation  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def plan(n, cell, f, f_y, alpha, seed):
+    sim = PrismSimulation(P.make_grid(n, n, 1, cell, cell, 2.0, 300.0, f, 2, 0.5, alpha, f_y=f_y))
+    i = sim.info
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    S = torch.randn((i.n_beams, i.ny_s, i.nx_s, 2), generator=g, device="cuda")
+    sim.load_smatrix(torch.view_as_complex(S))
+    return sim
+
+
+def close(got, ref, beams):
+    # both sum the same products in FP32 in another order: at most one rounding of 2^-24 per beam and per
+    # butterfly stage (two transforms of up to 7 stages, and the combinations), twice that for intensities
+    tol = 2.0 * (beams + 24) * 2.0 ** -24
+    err = np.linalg.norm(got.astype(np.float64) - ref) / np.linalg.norm(ref)
+    assert err <= tol, (err, tol)
+
+
+def raster(kind, cell, px, py, step):
+    x = np.arange(px) * step
+    y = np.arange(py) * step * 0.9
+    X, Y = np.meshgrid(x, y)
+    if kind == "wrap":       # across both cell edges, from negative positions
+        X, Y = X - 3.3 * step, Y + cell - 1.7 * step
+    elif kind == "serpentine":
+        X[1::2] = X[1::2, ::-1]
+    elif kind == "skew":     # every row shifted, rows in falling order
+        X = X + np.arange(py)[:, None] * 0.37 + 2.0 * cell
+        Y = Y[::-1] - 5.0 * cell
+    return np.ascontiguousarray(X).ravel(), np.ascontiguousarray(Y).ravel()
+
+
+@pytest.mark.parametrize("n,cell,f,f_y,alpha", [
+    (64, 8.0, 2, 0, 20.0),      # 16 x 16
+    (64, 8.0, 2, 1, 20.0),      # 16 x 32
+    (128, 12.8, 1, 4, 20.0),    # 64 x 16
+    (256, 16.0, 4, 0, 20.0),    # 32 x 32
+    (256, 16.0, 4, 2, 9.0),     # 32 x 64
+    (256, 12.5, 2, 0, 28.0),    # 64 x 64, 9 pairs of m: two chunks
+    (256, 16.0, 1, 0, 14.0),    # 128 x 128
+    (256, 16.0, 4, 0, 1.0),     # one beam
+])
+@pytest.mark.parametrize("kind,px,py,step", [("plain", 3, 5, 0.3), ("wrap", 33, 3, 0.21), ("serpentine", 9, 6, 0.05),
+                                             ("skew", 17, 9, 0.4), ("wrap", 7, 4, 2.7), ("plain", 64, 2, 0.11)])
+def test_rows_equal_the_general_scan(n, cell, f, f_y, alpha, kind, px, py, step):
+    sim = plan(n, cell, f, f_y, alpha, 5)
+    x0, y0 = raster(kind, cell, px, py, step)
+    probe = P.make_probe(20.0, 30.0, 1.0e6, 1.0e-3, -2.0e-3)
+    det = P.make_detector(0.0, 2.0, 40)
+    beams = sim.info.n_beams
+    got = sim.scan(probe, x0, y0, det, px=px, py=py).cpu().numpy()
+    ref = sim.scan(probe, x0, y0, det).cpu().numpy()  # one list of positions: y varies within it
+    close(got, ref, beams)
+    cb = sim.scan_cbed(probe, x0, y0, px=px, py=py).cpu().numpy()
+    close(cb, sim.scan_cbed(probe, x0, y0).cpu().numpy(), beams)
+    acc = torch.from_numpy(ref).cuda()
+    sim.scan_accumulate(probe, x0, y0, det, 0.5, acc, px=px, py=py)
+    close(acc.cpu().numpy(), 1.5 * ref, beams)
+    sim.close()
+
+
+@pytest.mark.parametrize("det", [(0.0, 400.0, 1), (3.0, 0.25, 400), (0.0, 1.0, 4096), (1.0e4, 1.0, 3)])
+def test_rows_bins(det):
+    # one bin over the whole window, more bins than pixels, lists longer than the windows, empty bins
+    sim = plan(256, 16.0, 4, 0, 20.0, 6)
+    x0, y0 = raster("wrap", 16.0, 11, 6, 0.3)
+    d = P.make_detector(*det)
+    got = sim.scan(P.make_probe(20.0), x0, y0, d, px=11, py=6).cpu().numpy()
+    ref = sim.scan(P.make_probe(20.0), x0, y0, d).cpu().numpy()
+    if ref.any():
+        close(got, ref, sim.info.n_beams)
+    else:
+        assert not got.any()
+    sim.close()
+
+
+def test_rows_partition_and_repeat_bitwise():
+    # a probe's result does not depend on the rows scanned with it (bands of rows, single rows), and a
+    # second scan on the same plan repeats it; a smaller scan in between changes nothing
+    sim = plan(256, 16.0, 4, 0, 20.0, 7)
+    x0, y0 = raster("plain", 16.0, 40, 23, 0.3)
+    probe, det = P.make_probe(20.0, 12.0), P.make_detector(0.0, 1.0, 100)
+    whole = sim.scan(probe, x0, y0, det, px=40, py=23).cpu().numpy()
+    sim.scan(probe, x0[:6], y0[:6], det, px=6, py=1)
+    assert np.array_equal(sim.scan(probe, x0, y0, det, px=40, py=23).cpu().numpy(), whole)
+    for rows in (1, 5):
+        for r in range(0, 23, rows):
+            k = min(rows, 23 - r)
+            part = sim.scan(probe, x0[r * 40:(r + k) * 40], y0[r * 40:(r + k) * 40], det, px=40, py=k).cpu().numpy()
+            assert np.array_equal(part, whole[r * 40:(r + k) * 40])
+    sim.close()
