@@ -794,30 +794,13 @@ static ColArgs col_args(const GridTables &T, float2 *wave, const float2 *prop_x,
 
 static int build_launches(prism_plan *P, const float *V_dev, int per = 0);
 
-// the column pass's launch shape when none is tuned or pinned: at N = 1024 the TMA-staged shape of
-// 4 columns per CTA, 3 CTAs per SM (the fastest there: 0.275 ms per launch on the 1024^2 carbon
-// workload, against 0.293 with 8 columns and 0.320 for cp.async staging), when the plan holds the
-// tensor maps of its wave; otherwise the default launcher (-1)
-// In a batch graph with parallel branches the passes of different cells share the SMs, and a shape
-// that fills an SM by itself (3 CTAs of 66 KB and 168 x 128 registers) leaves no room for the
-// other branches' kernels: there the 8-column TMA shape (one 131 KB CTA per SM) is the default, and
-// the autotuner skips the SM-filling shapes (64 uneven cells, 4 branches: 2.78 s per run with them,
-// 2.25 s without).
-static int col_default_shape(const prism_plan *P) {
-    if (P->g.ny != 1024 || !P->wave_map_ok) return -1;
-    const int v = tune_col_tma_shape(P->shared_sms ? 8 : 4);
-    return v >= 0 && tune_shape_valid(PRISM_TUNE_COL, 1024, v) ? v : -1;
+// the passes' launch shapes for nb beams when none is tuned or pinned (tune_col_default, tune_row_default)
+static int col_default_shape(const prism_plan *P, int nb) {
+    const int kept = P->T.kx_half > 0 ? 2 * P->T.kx_half : P->g.nx;
+    return tune_col_default(P->g.ny, (long long)kept * nb, P->wave_map_ok, P->shared_sms);
 }
-
-// the row pass's launch shape when none is tuned or pinned: at N = 1024, 384 threads (12 warps per
-// SM) with the next row's two kept quarters staged by bulk TMA copies (0.292 ms per launch on the
-// 1024^2 carbon workload, against 0.315 for 256 threads staged by cp.async and 0.333 for 128 threads
-// unstaged); in a batch graph, whose branches share the SMs, the default launcher's smaller CTAs
-// (this shape holds 163 KB of shared memory per CTA)
-static int row_default_shape(const prism_plan *P) {
-    if (P->g.nx != 1024 || P->shared_sms) return -1;
-    const int v = tune_row_find(384, false, true);
-    return v >= 0 && tune_shape_valid(PRISM_TUNE_ROW, 1024, v) ? v : -1;
+static int row_default_shape(const prism_plan *P, int nb) {
+    return tune_row_default(P->g.nx, (long long)P->g.ny * nb, P->shared_sms);
 }
 
 // the plan's wave stack in the column arguments of its build and autotuner launches
@@ -884,7 +867,7 @@ static int build_launches(prism_plan *P, const float *V_dev, int per) {
                 ra.trans = P->t + (size_t)p * px;
                 ra.n_rows = nb * g.ny;
                 ra.beam0 = b0;
-                const int rs = P->tune_shape[0] >= 0 ? P->tune_shape[0] : row_default_shape(P);
+                const int rs = P->tune_shape[0] >= 0 ? P->tune_shape[0] : row_default_shape(P, nb);
                 rc = plan_launch(P, PRISM_K_ROW, [&] {
                     return rs >= 0 ? launch_row_shape(g.nx, rs, ra, P->stream) : launch_row(g.nx, ROW_STD, ra, P->stream);
                 });
@@ -897,7 +880,7 @@ static int build_launches(prism_plan *P, const float *V_dev, int per) {
             ca.kx_half = P->T.kx_half;
             ca.band4 = P->T.band4;
             col_wave_map(P, ca);
-            const int cs = P->tune_shape[1] >= 0 ? P->tune_shape[1] : col_default_shape(P);
+            const int cs = P->tune_shape[1] >= 0 ? P->tune_shape[1] : col_default_shape(P, nb);
             rc = plan_launch(P, PRISM_K_COL, [&] {
                 return cs >= 0 ? launch_col_shape(g.ny, cs, ca, P->stream) : launch_col(g.ny, COL_STD, ca, P->stream);
             });
@@ -1347,9 +1330,9 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
     if ((rc = A.upload(&d_off, off))) return done(rc);
     if ((rc = A.upload(&d_idx, idx))) return done(rc);
     if ((rc = A.alloc((void **)&pos, (size_t)Pn * 2 * sizeof(double)))) return done(rc);
-    // the column passes between slices as in a plan's build: at 1024^2 the TMA-staged shape (tiles
-    // loaded and stored by TMA through tensor maps of this call's wave buffer); their bounded waits
-    // report to an error word that turns the affected bins into NaN
+    // the column passes between slices as in a plan's build: from 256^2 to 1024^2 the TMA-staged shapes
+    // where they are the default (tiles loaded and stored by TMA through tensor maps of this call's wave
+    // buffer); their bounded waits report to an error word that turns the affected bins into NaN
     int *err = nullptr;
     if ((rc = A.alloc((void **)&err, 16))) return done(rc);
     {
@@ -1360,9 +1343,7 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
         }
     }
     CUtensorMap map8, map4, out8, out4;
-    const int col_tma = ny == 1024 ? tune_col_tma_shape(4) : -1;
-    const bool maps_ok =
-        col_tma >= 0 && tune_shape_valid(PRISM_TUNE_COL, ny, col_tma) && encode_wave_maps(map8, map4, out8, out4, wave, nx, ny, Pb);
+    const bool maps_ok = (ny == 256 || ny == 512 || ny == 1024) && encode_wave_maps(map8, map4, out8, out4, wave, nx, ny, Pb);
     {
         // the probe phase uses r0 - h tan(theta) (zero without tilt)
         std::vector<double> xy((size_t)Pn * 2);
@@ -1421,14 +1402,17 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
             // columns the row passes skip) and writes every intensity
             ca.kx_half = p + 1 == g.n_slices ? 0 : kx_half;
             ca.band4 = T.band4;
-            if (p + 1 < g.n_slices && maps_ok) {
-                ca.wave_map = map8;
-                ca.wave_map4 = map4;
-                ca.out_map = out8;
-                ca.out_map4 = out4;
-                ca.wave_map_ok = 1;
-                ca.err = err;
-                if ((rc = check(launch_col_shape(ny, col_tma, ca, st), "column pass"))) return done(rc);
+            const int cs = p + 1 < g.n_slices ? tune_col_default(ny, (long long)(kx_half > 0 ? 2 * kx_half : nx) * nb, maps_ok, false) : -1;
+            if (cs >= 0) {
+                if (maps_ok) {
+                    ca.wave_map = map8;
+                    ca.wave_map4 = map4;
+                    ca.out_map = out8;
+                    ca.out_map4 = out4;
+                    ca.wave_map_ok = 1;
+                    ca.err = err;
+                }
+                if ((rc = check(launch_col_shape(ny, cs, ca, st), "column pass"))) return done(rc);
             } else if ((rc = check(launch_col(ny, p + 1 == g.n_slices ? COL_DETECT : COL_STD, ca, st), "column pass"))) {
                 return done(rc);
             }
@@ -1817,7 +1801,7 @@ extern "C" int prism_plan_tune_result(const prism_plan *P, int kind, prism_tune_
     const int n = kind == 0 ? P->g.nx : P->g.ny;
     out->n_shapes = std::min(tune_shapes(kind), PRISM_TUNE_MAX_SHAPES);
     out->chosen = P->tune_shape[kind];
-    const int dc = kind == PRISM_TUNE_COL ? col_default_shape(P) : row_default_shape(P);
+    const int dc = kind == PRISM_TUNE_COL ? col_default_shape(P, P->batch) : row_default_shape(P, P->batch);
     out->default_shape = dc >= 0 ? dc : tune_shape_valid(kind, n, tune_default_shape(kind, n)) ? tune_default_shape(kind, n) : -1;
     for (int v = 0; v < PRISM_TUNE_MAX_SHAPES; ++v) out->ms[v] = P->tuned[kind] ? P->tune_ms[kind][v] : -1.0;
     return PRISM_OK;

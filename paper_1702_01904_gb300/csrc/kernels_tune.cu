@@ -86,24 +86,58 @@ bool tune_shape_needs_map(int kind, int v) { return kind == 1 && v >= 0 && v < N
 
 bool tune_shape_fills_sm(int kind, int v) { return kind == 1 && v >= 0 && v < N_COL && COL_SHAPES[v].mb >= 3; }
 
-int tune_row_find(int thr, bool stg, bool tma) {
+static int tune_row_find(int thr, bool stg, bool tma) {
     for (int v = 0; v < N_ROW; ++v)
         if (ROW_SHAPES[v].a == thr && ROW_SHAPES[v].stg == stg && ROW_SHAPES[v].tma == tma && ROW_SHAPES[v].rv == 0) return v;
     return -1;
 }
 
-cudaError_t launch_row_std(int nx, const RowArgs &a, cudaStream_t s) {
-    if (nx == 1024) {
-        const int v = tune_row_find(384, false, true);
-        if (v >= 0 && tune_row_valid(1024, v)) return tune_row_launch(1024, v, a, s);
-    }
-    return launch_row(nx, ROW_STD, a, s);
+// The row pass's launch shape when none is tuned or pinned (-1: the default launcher).  N = 1024: 384
+// threads (12 warps per SM) with the next row's two kept quarters staged by bulk TMA copies (0.292 ms
+// per launch for 129 beams, against 0.315 for 256 threads staged by cp.async and 0.333 for 128 threads
+// unstaged).  N = 512: 384 threads staged by cp.async from 16 384 rows on (213 beams: 123 us against
+// 132 for 128 threads unstaged; 829 beams 446 against 490; 49 beams 33.4 against 33.5; with 13 beams,
+// 6656 rows, the small CTAs are faster, 12.9 against 14.0).  In a batch graph, whose branches share the
+// SMs, the default launcher's smaller CTAs (the 1024 shape holds 163 KB of shared memory per CTA).
+int tune_row_default(int nx, long long rows, bool shared) {
+    if (shared) return -1;
+    const int v = nx == 1024 ? tune_row_find(384, false, true) : nx == 512 && rows >= 16384 ? tune_row_find(384, true, false) : -1;
+    return v >= 0 && tune_row_valid(nx, v) ? v : -1;
 }
 
-int tune_col_tma_shape(int w) {
+cudaError_t launch_row_std(int nx, const RowArgs &a, cudaStream_t s) {
+    const int v = tune_row_default(nx, a.n_rows, false);
+    return v >= 0 ? tune_row_launch(nx, v, a, s) : launch_row(nx, ROW_STD, a, s);
+}
+
+static int tune_col_find(int w, bool stg, bool tma) {
     for (int v = 0; v < N_COL; ++v)
-        if (COL_SHAPES[v].tma && COL_SHAPES[v].a == w && COL_SHAPES[v].rv == 0) return v;
+        if (COL_SHAPES[v].tma == tma && COL_SHAPES[v].a == w && COL_SHAPES[v].stg == stg && COL_SHAPES[v].rv == 0 &&
+            (tma || COL_SHAPES[v].mb == 0))
+            return v;
     return -1;
+}
+
+// The column pass's launch shape when none is tuned or pinned (-1: the default launcher), for `cols`
+// columns in all and with (maps) or without tensor maps of the wave stack.  N = 1024: 4 columns per CTA
+// staged by TMA, 3 CTAs per SM (0.200 ms for 129 beams, against 0.293 for 8 columns by TMA and 0.320
+// by cp.async).  N = 512: the same from 8192 columns on (213 beams, 54 528 columns: 88 us against 125 for
+// 16 columns by cp.async; 49 beams 24.2 against 31.2), below that 8 columns unstaged (13 beams, 3328
+// columns: 10.8 against 12.4 by TMA and 12.8).  N = 256: 8 columns by TMA from 16 384 columns on (829
+// beams, 106 112 columns: 82 us against 110 for 16 columns by cp.async; 213 beams 23.1 against 30.9),
+// below that 8 columns unstaged (49 beams, 6272 columns: 8.7 against 10.8 for either).
+// In a batch graph with parallel branches the passes of different cells share the SMs, and a shape that
+// fills an SM by itself (3 CTAs of 66 KB and 168 x 128 registers) leaves no room for the other branches'
+// kernels: there the default is 8 columns by TMA at N = 1024 (one 131 KB CTA per SM) and the default
+// launcher elsewhere, and the autotuner skips the SM-filling shapes (64 uneven cells, 4 branches: 2.78 s
+// per run with them, 2.25 s without).
+int tune_col_default(int ny, long long cols, bool maps, bool shared) {
+    int v = -1;
+    if (ny == 1024) v = maps ? tune_col_find(shared ? 8 : 4, false, true) : -1;
+    else if (shared) v = -1;
+    else if (ny == 512) v = maps && cols >= 8192 ? tune_col_find(4, false, true) : tune_col_find(8, false, false);
+    else if (ny == 256) v = maps && cols >= 16384 ? tune_col_find(8, false, true) : tune_col_find(8, false, false);
+    return v >= 0 && tune_shape_valid(1, ny, v) ? v : -1;
 }
 
 bool tune_row_valid(int n, int v) {

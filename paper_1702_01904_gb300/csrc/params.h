@@ -229,13 +229,14 @@ bool tune_shape_valid(int kind, int n, int v);
 bool tune_shape_needs_map(int kind, int v);  // the shape stages through TMA (ColArgs::wave_map)
 int tune_shape_fft_variant(int kind, int v);  // its FFT radix variant (DftSplit), -1 if unknown
 int tune_default_fft_variant(int n);          // the radix variant of the default launchers at N
-int tune_col_tma_shape(int w);                // the TMA-staged column shape of w columns per CTA, or -1
-int tune_row_find(int thr, bool stg, bool tma);  // the row shape of thr threads per CTA and that staging, or -1
+// the shape of a standard pass when none is tuned or pinned (-1: the default launcher): rows of all
+// waves; columns of all waves, whether tensor maps of the waves are at hand; shared: beside other
+// kernels on the same SMs
+int tune_row_default(int nx, long long rows, bool shared);
+int tune_col_default(int ny, long long cols, bool maps, bool shared);
 bool tune_shape_fills_sm(int kind, int v);    // 3 or more CTAs per SM, each with a third of its resources
 cudaError_t launch_row_shape(int nx, int v, const RowArgs &a, cudaStream_t s);
-// the standard row pass of a multislice scan: at nx = 1024 the 384-thread shape with the next row's
-// kept quarters staged by bulk TMA copies (the fastest there), elsewhere the default launcher; every
-// shape computes the same rows
+// the standard row pass in its default shape (tune_row_default); every shape computes the same rows
 cudaError_t launch_row_std(int nx, const RowArgs &a, cudaStream_t s);
 cudaError_t launch_col_shape(int ny, int v, const ColArgs &a, cudaStream_t s);
 // smallest scan-window / FFT sizes the kernels are instantiated for
