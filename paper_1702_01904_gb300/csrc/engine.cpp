@@ -112,11 +112,12 @@ static Tw64 make_tw64() {
     return t;
 }
 
-// inter-stage twiddles of a two-level FFT with split (A, B): table[k1 * B + n2] = W_N^{n2 k1}
-static std::vector<float2> stage_table(int N, int A, int B) {
+// inter-stage twiddles of a two-level FFT with split (A, B): table[k1 * B + n2] = W_N^{n2 k1}, or, for
+// the passes' transforms on signed residues (fft.cuh), W_N^{s(n2) k1} with s(n2) in [-B/2, B/2)
+static std::vector<float2> stage_table(int N, int A, int B, bool sg = false) {
     std::vector<float2> t((size_t)A * B);
     for (int k1 = 0; k1 < A; ++k1)
-        for (int n2 = 0; n2 < B; ++n2) t[(size_t)k1 * B + n2] = wN((long long)n2 * k1, N);
+        for (int n2 = 0; n2 < B; ++n2) t[(size_t)k1 * B + n2] = wN((long long)(sg ? signed_index(n2, B) : n2) * k1, N);
     return t;
 }
 
@@ -279,8 +280,8 @@ static int build_grid_tables(const prism_grid *g, GridTables &T) {
     T.twr_f = stage_table(T.nx, a1, a2);
     T.twr_i = stage_table(T.nx, a2, a1);
     fft_split(T.ny, &a1, &a2);
-    T.twc_f = stage_table(T.ny, a1, a2);
-    T.twc_i = stage_table(T.ny, a2, a1);
+    T.twc_f = stage_table(T.ny, a1, a2, true);
+    T.twc_i = stage_table(T.ny, a2, a1, true);
     return PRISM_OK;
 }
 
@@ -1332,8 +1333,9 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
     if ((rc = A.alloc((void **)&pos, (size_t)Pn * 2 * sizeof(double)))) return done(rc);
     // the column passes between slices as in a plan's build: from 256^2 to 1024^2 the TMA-staged shapes
     // where they are the default (tiles loaded and stored by TMA through tensor maps of this call's wave
-    // buffer); their bounded waits report to an error word that turns the affected bins into NaN
-    int *err = nullptr;
+    // buffer), their tiles from a counter; their bounded waits report to an error word that turns the
+    // affected bins into NaN
+    int *err = nullptr;  // error word, then the tile counter (two ints, zero between launches)
     if ((rc = A.alloc((void **)&err, 16))) return done(rc);
     {
         const cudaError_t e = cudaMemsetAsync(err, 0, 16, st);
@@ -1410,6 +1412,7 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
                     ca.out_map = out8;
                     ca.out_map4 = out4;
                     ca.wave_map_ok = 1;
+                    ca.tile_ctr = err + 1;
                     ca.err = err;
                 }
                 if ((rc = check(launch_col_shape(ny, cs, ca, st), "column pass"))) return done(rc);

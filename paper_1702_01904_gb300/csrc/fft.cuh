@@ -17,6 +17,17 @@
 // A forward transform with split (A, B) leaves its output in exactly the input layout of an
 // inverse transform with split (B, A), and vice versa, so FFT -> pointwise -> IFFT chains need no
 // data movement between transforms.
+//
+// Signed residues.  n2 and k1 may be taken as any representatives of their residues.  With k1 in
+// [-N1/2, N1/2) (SGO) the twiddles of k1 and -k1 are conjugates of each other, so a lane reads 16 of them
+// instead of 31 (N1 = 32); SGI takes n2 in [-N2/2, N2/2), the input layout that matches such an output.
+// With s(n) = n below half, else n - length:
+//   input : reg n1*J + j  holds element  N2*n1 + s(t + T*j)   (mod N)
+//   output: reg k2*I + i  holds element  s(t + T*i) + N1*k2   (mod N)
+// Used by the column passes (both transforms): their tile loop waits on shared memory, and half of the
+// twiddle reads are a quarter of its reads (203 -> 195 us per 129-beam launch at 1024^2 with tiles from
+// the counter).  Not by the row passes: there the band |k| < N/4 no longer ends at a register's edge,
+// which costs 5 % more instructions where the FMA pipe is the limit (93 -> 97 us on a 37-beam launch).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -358,8 +369,9 @@ struct NoHook {
 // table laid out [k1][n2] = W_N^{n2 k1} (forward sign; the inverse conjugates it); kernels keep
 // it in shared memory (lanes read consecutive n2: conflict-free).  `Ex` is the exchange:
 // write(k1, n2, v), read(k1, n2), sync().
-// V: split variant of the register DFTs (DftSplit)
-template <int N1, int N2, bool INV, int V = 0>
+// V: split variant of the register DFTs (DftSplit); SGI: signed residues n2 (the table is then
+// W_N^{s(n2) k1}), SGO: signed residues k1 (only the table's rows k1 <= N1/2 are read, kTwiddles entries)
+template <int N1, int N2, bool INV, int V = 0, bool SGI = false, bool SGO = false>
 struct BlockFft {
     static constexpr int SPLIT1 = N1, SPLIT2 = N2;  // first-stage, second-stage DFT lengths
     static constexpr int N = N1 * N2;
@@ -367,6 +379,13 @@ struct BlockFft {
     static constexpr int T = N / E;
     static constexpr int J = E / N1;
     static constexpr int I = E / N2;
+    static constexpr int kTwiddles = SGO ? (N1 / 2 + 1) * N2 : N1 * N2;
+
+    // x times the twiddle of k1 >= 1 from the table's value: rows past N1/2 take the conjugate of -k1's
+    template <int K1>
+    __device__ __forceinline__ static float2 twiddled(float2 x, float2 w) {
+        return (SGO && K1 >= N1 / 2) != INV ? cmulc(x, w) : cmul(x, w);
+    }
 
     // GTW: where the twiddle table is and how it is read: TW_SMEM (shared memory, every twiddle
     // loaded before the first exchange store), TW_GLOBAL (global memory through the read-only path,
@@ -386,15 +405,16 @@ struct BlockFft {
         if constexpr (GTW == TW_SMEM) {
             // shared-memory table: all twiddle loads before any exchange store (the table and the
             // exchange share the address space, and this order lets the loads issue back to back)
-#pragma unroll
-            for (int j = 0; j < J; ++j) {
+            static_for<J>([&](auto jc) {
+                constexpr int j = decltype(jc)::value;
                 const int n2 = t + T * j;
-#pragma unroll
-                for (int k1 = 1; k1 < N1; ++k1) {
+                static_for<SGO ? N1 / 2 : N1 - 1>([&](auto kc) {
+                    constexpr int k1 = decltype(kc)::value + 1;
                     const float2 w = stw[k1 * N2 + n2];
-                    x[k1 * J + j] = INV ? cmulc(x[k1 * J + j], w) : cmul(x[k1 * J + j], w);
-                }
-            }
+                    x[k1 * J + j] = twiddled<k1>(x[k1 * J + j], w);
+                    if constexpr (SGO && k1 < N1 / 2) x[(N1 - k1) * J + j] = twiddled<N1 - k1>(x[(N1 - k1) * J + j], w);
+                });
+            });
             if constexpr (LEAD) ex.sync();  // previous readers of the exchange are done
 #pragma unroll
             for (int j = 0; j < J; ++j) {
@@ -405,19 +425,17 @@ struct BlockFft {
         } else {
             // interleave load, multiply and store (TW_GLOBAL: read-only path, L1-resident)
             if constexpr (LEAD) ex.sync();
-#pragma unroll
-            for (int j = 0; j < J; ++j) {
+            static_for<J>([&](auto jc) {
+                constexpr int j = decltype(jc)::value;
                 const int n2 = t + T * j;
-#pragma unroll
-                for (int k1 = 0; k1 < N1; ++k1) {
-                    float2 v = x[k1 * J + j];
-                    if (k1 != 0) {
-                        const float2 w = GTW == TW_GLOBAL ? __ldg(stw + k1 * N2 + n2) : stw[k1 * N2 + n2];
-                        v = INV ? cmulc(v, w) : cmul(v, w);
-                    }
-                    ex.write(k1, n2, v);
-                }
-            }
+                ex.write(0, n2, x[j]);
+                static_for<SGO ? N1 / 2 : N1 - 1>([&](auto kc) {
+                    constexpr int k1 = decltype(kc)::value + 1;
+                    const float2 w = GTW == TW_GLOBAL ? __ldg(stw + k1 * N2 + n2) : stw[k1 * N2 + n2];
+                    ex.write(k1, n2, twiddled<k1>(x[k1 * J + j], w));
+                    if constexpr (SGO && k1 < N1 / 2) ex.write(N1 - k1, n2, twiddled<N1 - k1>(x[(N1 - k1) * J + j], w));
+                });
+            });
         }
         ex.sync();
         hook();
@@ -431,9 +449,20 @@ struct BlockFft {
         for (int i = 0; i < I; ++i) Dft<N2, I, INV, 0, V>::run(x + i, tw);
     }
 
+    // s(t + T j) of L residues, G = L / T of them per lane (with G > 1 a lane's j-th lies in one half)
+    template <bool SG, int L, int G>
+    __host__ __device__ __forceinline__ static constexpr int residue(int t, int j) {
+        return !SG ? t + T * j : G > 1 ? t + T * j - (2 * T * j >= L ? L : 0) : t < L / 2 ? t : t - L;
+    }
     // element index held in register r (input / output layouts)
-    __host__ __device__ __forceinline__ static constexpr int in_elem(int r, int t) { return N2 * (r / J) + t + T * (r % J); }
-    __host__ __device__ __forceinline__ static constexpr int out_elem(int r, int t) { return t + T * (r % I) + N1 * (r / I); }
+    __host__ __device__ __forceinline__ static constexpr int in_elem(int r, int t) {
+        const int s = residue<SGI, N2, J>(t, r % J);
+        return SGI && r / J == 0 && s < 0 ? N + s : N2 * (r / J) + s;
+    }
+    __host__ __device__ __forceinline__ static constexpr int out_elem(int r, int t) {
+        const int s = residue<SGO, N1, I>(t, r % I);
+        return SGO && r / I == 0 && s < 0 ? N + s : s + N1 * (r / I);
+    }
 };
 
 // Band classes of the registers of a transform of length N for the band |k| < N/4 (FFT order):
@@ -465,10 +494,15 @@ __host__ __device__ constexpr unsigned long long band_zero_mask(bool input) {
     return m;
 }
 
+template <int N, int V = 0, bool SGI = false, bool SGO = false>
+using FwdFft = BlockFft<FftShape<N>::N1, FftShape<N>::N2, false, V, SGI, SGO>;
+template <int N, int V = 0, bool SGI = false, bool SGO = false>
+using InvFft = BlockFft<FftShape<N>::N2, FftShape<N>::N1, true, V, SGI, SGO>;
+// the column passes' transforms
 template <int N, int V = 0>
-using FwdFft = BlockFft<FftShape<N>::N1, FftShape<N>::N2, false, V>;
+using FwdCol = FwdFft<N, V, true, true>;
 template <int N, int V = 0>
-using InvFft = BlockFft<FftShape<N>::N2, FftShape<N>::N1, true, V>;
+using InvCol = InvFft<N, V, true, true>;
 
 // Exchange for transforms held by T consecutive lanes of one warp (T <= 32); each transform
 // owns N1*(N2+1) float2 of shared memory (the +1 pad keeps stage-2 reads at two wavefronts).

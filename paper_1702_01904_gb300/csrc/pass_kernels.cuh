@@ -381,7 +381,9 @@ struct ColCfg {
     static constexpr int EX = ColExSize<NY, W>::value;
     static_assert(EX >= NY * W, "the exchange buffer holds a whole tile (TMA stores)");
     static_assert(!TM || (FS::T % (32 / W) == 0 && FS::T * W >= 32), "TMA stores: whole warps of lanes per column");
-    static constexpr size_t SMEM = (size_t)((SMEM_TW ? NY : 0) + (STAGE ? NY * W : 0) + EX) * sizeof(float2);
+    static constexpr int TWF2 = SMEM_TW ? FwdCol<NY>::kTwiddles : 0;
+    static_assert(TWF2 % 16 == 0, "128-byte aligned tiles");
+    static constexpr size_t SMEM = (size_t)(TWF2 + (STAGE ? NY * W : 0) + EX) * sizeof(float2);
 };
 
 // TMA staging gives up after this many SM cycles (about a second) and reports it in the error word
@@ -394,8 +396,8 @@ template <int NY, int MODE, int WC = col_default_w<NY>(), bool STG = true, int M
 __global__ void __launch_bounds__(ColCfg<NY, WC, STG, MB, TM>::THREADS, ColCfg<NY, WC, STG, MB, TM>::MINB) k_col(const __grid_constant__ ColArgs a) {
     using C = ColCfg<NY, WC, STG, MB, TM>;
     using FS = FftShape<NY>;
-    using Fwd = FwdFft<NY, RV & 1>;
-    using Inv = InvFft<NY, (RV >> 1) & 1>;
+    using Fwd = FwdCol<NY, RV & 1>;
+    using Inv = InvCol<NY, (RV >> 1) & 1>;
     constexpr int W = C::W, E = FS::E, THREADS = C::THREADS;
     extern __shared__ __align__(128) float2 smem_c[];
     float2 *smem = smem_c;
@@ -413,12 +415,12 @@ __global__ void __launch_bounds__(ColCfg<NY, WC, STG, MB, TM>::THREADS, ColCfg<N
     const float2 *twf = a.tw_fwd, *twi = a.tw_inv;
     if constexpr (C::SMEM_TW) {
         float2 *tws = smem;
-        for (int i = threadIdx.x; i < NY; i += THREADS) tws[i] = a.tw_fwd[i];
+        for (int i = threadIdx.x; i < C::TWF2; i += THREADS) tws[i] = a.tw_fwd[i];
         __syncthreads();
         twf = tws;
         twi = tws;  // the square split's inverse table holds the same values
     }
-    float2 *stg = smem + (C::SMEM_TW ? NY : 0);
+    float2 *stg = smem + C::TWF2;
     float2 *exb = stg + (C::STAGE ? NY * W : 0);
     const int c = threadIdx.x % W, t = threadIdx.x / W, lane = threadIdx.x & 31;
     ColExchange<FS::N1, FS::N2, W> exF{exb, c};
@@ -607,15 +609,19 @@ __global__ void __launch_bounds__(ColCfg<NY, WC, STG, MB, TM>::THREADS, ColCfg<N
             for (int r = 0; r < E; ++r) v[r] = cscale(v[r], a.probe_scale);
         }
         if constexpr (C::TMA) {
-            // result register r of lane t is row t + T r: it goes back to the exchange slot (t, r) that
-            // this thread alone read in the inverse transform's second stage, so no barrier is needed
+            // result register r of lane t is row s(t) + T r (mod NY), that is t + T r or, for the upper half
+            // of the lanes, t + T (r - 1): it goes back to the exchange slot (t, r) or (t, r - 1), of the E
+            // that this thread alone read in the inverse transform's second stage, so no barrier is needed
             // before the writes; the slots of a warp's lanes (T / (32 / W) consecutive t) are one
             // contiguous box of the store map, [t][E + 1][W], which lane 0 stores once the warp's
             // writes are visible to the async proxy
-            static_assert(Inv::I == 1 && Inv::SPLIT1 == FS::T && Inv::SPLIT2 == E, "result row = t + T r");
+            static_assert(Inv::I == 1 && Inv::SPLIT1 == FS::T && Inv::SPLIT2 == E, "result row = s(t) + T r");
             constexpr int TPW = 32 / W;  // lanes t per warp
+            const int up = t >= FS::T / 2;
+            float2 *xo = exb + (t * (E + 1) - up) * W + c;
+            xo[up ? E * W : 0] = v[0];
 #pragma unroll
-            for (int r = 0; r < E; ++r) exb[(t * (E + 1) + r) * W + c] = v[r];
+            for (int r = 1; r < E; ++r) xo[r * W] = v[r];
             tc::fence_proxy_async();  // the generic writes before the async-proxy reads
             __syncwarp();
             if (lane == 0 && valid) {
