@@ -75,7 +75,8 @@ extern "C" {
  *                PRISM_PRECISION_FP16X2: the same with every S value and coefficient stored as an
  *                FP16 value plus the FP16 rounding of its remainder and three tensor-core products
  *                per step (value x value + value x remainder + remainder x value), FP32-class
- *                accuracy with the storage of FP32.  The build
+ *                accuracy with the storage of FP32. (Rasters whose rows of 3 or more probes each share
+ *                one y are summed by rows in FP32 from the unpacked values instead.)  The build
  *                (transmission, FFTs, propagator) is FP32 in every mode.  Ignored by
  *                multislice_scan_run.  Zero-initialised structs select FP32.
  *   f_y          interpolation factor along y when it differs from f (f is then the factor along

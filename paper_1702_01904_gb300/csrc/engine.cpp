@@ -416,6 +416,8 @@ struct prism_plan {
     int rows_m = 0, rows_maxn = 0;
     float2 *rows_w = nullptr;  // sums over n of the raster-row scan
     size_t rows_cap = 0;
+    float2 *rows_s = nullptr;  // what the windows reach of a value + remainder S-matrix, unpacked
+    size_t rows_s_cap = 0;
     // grown on demand
     double *pos = nullptr;
     size_t pos_cap = 0;
@@ -940,17 +942,19 @@ extern "C" int prism_build_smatrix_host(prism_plan *P, const float *V_host) {
 }
 
 // ------------------------------------------------------------------ scan
-// Whether the scan goes by raster rows (scan_rows.cuh), and its geometry: FP32 S-matrix, every row of
-// the raster on one y, rows of 3 probes or more, and few enough columns under the rows' windows.  A row's
-// sums cost one product per beam and column reached, then each probe one per distinct m and window pixel;
-// in blocks (scan_gemm.cuh) each probe costs one per beam and window pixel.  Measured over windows of 32
-// to 128 pixels, 49 to 529 beams, steps of 0.1 to 2 A and rasters of 2 x 2 to 64 x 64: 1.2 to 6.6 times
-// the speed of the blocks wherever the test below lets rows of 3 or more through, 0.84 to 1.06 times for
-// tall rasters of rows of 2.  Sets a.rows_lp > 0, the columns and the rows held at once, or leaves
-// a.rows_lp = 0.
+// Whether the scan goes by raster rows (scan_rows.cuh), and its geometry: FP32 or FP16 value + remainder
+// S-matrix, every row of the raster on one y, rows of 3 probes or more, and few enough columns under the
+// rows' windows.  A row's sums cost one product per beam and column reached, then each probe one per
+// distinct m and window pixel; in blocks (scan_gemm.cuh, scan_tc.cuh) each probe costs one per beam and
+// window pixel.  Measured over windows of 32 to 128 pixels, 49 to 529 beams, steps of 0.1 to 2 A and
+// rasters of 2 x 2 to 64 x 64: 1.2 to 6.6 times the speed of the FP32 blocks wherever the test below lets
+// rows of 3 or more through, 0.84 to 1.06 times for tall rasters of rows of 2.  The 16-bit precisions round
+// the coefficients of every beam and probe, which do not separate: they stay with the tensor cores.
+// Sets a.rows_lp > 0, the columns and the rows held at once, or leaves a.rows_lp = 0.
 static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) {
-    if (P->prec != PRISM_PRECISION_FP32 || sc->px < 3 || sc->py < 1) return;
-    double xmin = sc->x0[0], xmax = sc->x0[0];
+    const bool split = P->prec == PRISM_PRECISION_FP16X2;
+    if ((P->prec != PRISM_PRECISION_FP32 && !split) || sc->px < 3 || sc->py < 1) return;
+    double xmin = sc->x0[0], xmax = sc->x0[0], ymin = sc->y0[0], ymax = sc->y0[0];
     for (int r = 0; r < sc->py; ++r) {
         const double *x = sc->x0 + (size_t)r * sc->px, *y = sc->y0 + (size_t)r * sc->px;
         for (int i = 0; i < sc->px; ++i) {
@@ -958,26 +962,38 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
             xmin = std::min(xmin, x[i]);
             xmax = std::max(xmax, x[i]);
         }
+        ymin = std::min(ymin, y[0]);
+        ymax = std::max(ymax, y[0]);
     }
-    // columns from the first window's to the last one's, to whole runs of 16 (positions reach 2^28 pixels)
-    const long long first = (long long)std::floor(xmin / a.px_s + 0.5) - P->nw / 2;
-    const long long last = (long long)std::floor(xmax / a.px_s + 0.5) - P->nw / 2 + P->nw;
-    const long long g0 = first & ~15LL;
-    const long long reach = (last - g0 + 15) & ~15LL;
-    const int cols = (int)std::min<long long>(reach, P->nxs);
+    // columns from the first window's to the last one's, to whole runs of 16, and rows (positions reach
+    // 2^28 pixels); the whole grid where they reach around it
+    const auto reach = [](double lo, double hi, double px, int nw, int n, int align, int *origin) {
+        const long long first = ((long long)std::floor(lo / px + 0.5) - nw / 2) & ~(long long)(align - 1);
+        const long long last = (long long)std::floor(hi / px + 0.5) - nw / 2 + nw;
+        const long long len = (last - first + align - 1) & ~(long long)(align - 1);
+        *origin = len >= n ? 0 : (int)(((first % n) + n) % n);
+        return (int)std::min<long long>(len, n);
+    };
+    int gx = 0, gy = 0;
+    const int cols = reach(xmin, xmax, a.px_s, P->nw, P->nxs, 16, &gx);
+    const int rows = reach(ymin, ymax, a.py_s, P->nwy, P->nys, 1, &gy);
     const int planes = 2 * P->rows_m + 1;
     if ((double)cols * P->nbeams + (double)sc->px * P->nw * planes > 0.75 * (double)sc->px * P->nw * P->nbeams) return;
-    // rows held at once: no more memory than the blocks' window scratch would take (32 windows per
-    // block of 4 x 4, two blocks per SM at most, twice over for split blocks), and 384 MB (1.53 ms for the
-    // 200 x 200 probes of the carbon cell, two launches each of 100 rows; 192 MB: 1.64 ms, 640 MB: 1.52)
+    // memory for the rows held at once and the unpacked S-matrix: no more than the blocks' window scratch
+    // would take (32 windows per block of 4 x 4, two blocks per SM at most, twice over for split blocks),
+    // and 384 MB for the rows (1.53 ms for the 200 x 200 probes of the carbon cell, two launches each of
+    // 100 rows; 192 MB: 1.64 ms, 640 MB: 1.52)
     const size_t row = (size_t)P->nwy * planes * cols * sizeof(float2);
     const size_t blocks = ((size_t)sc->px + 3) / 4 * (((size_t)sc->py + 3) / 4);
-    const size_t most = std::min<size_t>(std::min<size_t>(blocks, 304) * 64 * P->nw * P->nwy * sizeof(float2), (size_t)384 << 20);
-    size_t chunk = std::min<size_t>(most / row, sc->py);
+    const size_t most = std::min<size_t>(blocks, 304) * 64 * P->nw * P->nwy * sizeof(float2);
+    const size_t unpacked = split ? (size_t)P->nbeams * rows * cols * sizeof(float2) : 0;
+    if (unpacked + row > most) return;
+    const size_t limit = std::min<size_t>(most - unpacked, (size_t)384 << 20);
+    size_t chunk = std::min<size_t>(limit / row, sc->py);
     if (chunk == 0) return;
     // in equal shares, to whole groups of 4
     chunk = ((size_t)sc->py + (sc->py + chunk - 1) / chunk - 1) / ((sc->py + chunk - 1) / chunk);
-    if (chunk % 4 && chunk < (size_t)sc->py && (chunk + 3) / 4 * 4 * row <= most) chunk = (chunk + 3) / 4 * 4;
+    if (chunk % 4 && chunk < (size_t)sc->py && (chunk + 3) / 4 * 4 * row <= limit) chunk = (chunk + 3) / 4 * 4;
     const int lp = scan_rows_lp(P->nw, P->nwy, P->rows_m, P->rows_maxn, a.n_fold16, sc->px, (int)chunk);
     if (lp <= 0) return;
     a.rows_lp = lp;
@@ -986,9 +1002,14 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
     a.m_off = P->m_off;
     a.m_beam = P->m_beam;
     a.m_qx = P->m_qx;
-    a.rows_g0 = cols == P->nxs ? 0 : (int)(((g0 % P->nxs) + P->nxs) % P->nxs);
+    a.rows_g0 = gx;
     a.rows_cols = cols;
     a.rows_chunk = (int)chunk;
+    a.rows_unpack = split ? 1 : 0;
+    a.rows_x0 = split ? gx : 0;
+    a.rows_y0 = split ? gy : 0;
+    a.rows_pitch = split ? cols : P->nxs;
+    a.rows_ry = split ? rows : P->nys;
 }
 
 static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_scan *sc, const prism_detector *det,
@@ -1148,6 +1169,11 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
         int rc = grow(P->arena, (void **)&P->rows_w, &P->rows_cap, wb);
         if (rc) return rc;
         a.rows_w = P->rows_w;
+        a.rows_src = P->S;
+        if (a.rows_unpack) {
+            if ((rc = grow(P->arena, (void **)&P->rows_s, &P->rows_s_cap, scan_rows_unpack_bytes(a)))) return rc;
+            a.rows_src = P->rows_s;
+        }
         *grid = 1;
         return PRISM_OK;
     }
@@ -1174,7 +1200,8 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
 static int scan_go(prism_plan *P, const ScanArgs &a, int grid) {
     if (a.rows_lp > 0) {
         const int rc = plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_rows(P->nw, P->nwy, a, P->stream); });
-        if (!rc) P->launches += 2 * ((a.scan_py + a.rows_chunk - 1) / a.rows_chunk) - 1;  // two kernels per chunk of rows
+        // two kernels per chunk of rows, and the unpacking
+        if (!rc) P->launches += 2 * ((a.scan_py + a.rows_chunk - 1) / a.rows_chunk) - 1 + a.rows_unpack;
         return rc;
     }
     if (P->prec == PRISM_PRECISION_FP32)

@@ -129,6 +129,10 @@ struct ScanArgs {
     float2 *rows_w;            // [rows_chunk][nw_y][2 M + 1][rows_cols] transformed sums over n
     int rows_g0, rows_cols;    // columns held: rows_g0 ... rows_g0 + rows_cols - 1 (mod nx_s), multiples of 16
     int rows_chunk;            // raster rows whose sums are held at once
+    const float2 *rows_src;    // the beams' values under the windows, [B][rows_ry][rows_pitch] from pixel
+    int rows_x0, rows_y0;      // (rows_x0, rows_y0) on (mod the stored grid): S itself, or (rows_unpack) the
+    int rows_pitch, rows_ry;   // reach of the windows unpacked from the value + remainder rows of S16
+    int rows_unpack;
     int rows_lp;               // probes per CTA
     int rows_0, rows_n;        // set per launch: first raster row, raster rows
     const uint16_t *fold16;    // the bins over the quadrant 0 <= kx <= nw_x/2, 0 <= ky <= nw_y/2: CSR offsets
@@ -198,6 +202,7 @@ size_t scan_gemm_cnt_bytes(int grid);
 // the raster-row scan (scan_rows.cuh): probes per CTA for rows of px probes
 // and so many 16-bit entries of bin lists (0: these windows, beams
 // or sizes are not for it), launch
+size_t scan_rows_unpack_bytes(const ScanArgs &a);  // bytes of rows_src where it is unpacked
 int scan_rows_lp(int nwx, int nwy, int m, int max_beams, int lists, int px, int rows);
 cudaError_t launch_scan_rows(int nwx, int nwy, const ScanArgs &a, cudaStream_t s);
 cudaError_t launch_shift(const ShiftArgs &a, cudaStream_t s);

@@ -11,7 +11,9 @@
 // transform commutes with the sum over m and with the choice of window columns (the window rows are
 // the row's), so it is made on A_m and B_m once per raster row instead of once per probe:
 //   k_rows_sum     per (4 raster rows, 16 columns, pair +-m): T, A, B, their column transforms, written
-//                  to W[row][ky][plane][column] (planes T_0, A_1, B_1, A_2, ...);
+//                  to W[row][ky][plane][column] (planes T_0, A_1, B_1, A_2, ...).
+//                  S comes beam by beam: the FP32 S-matrix itself, or what the windows reach of an FP16
+//                  value + remainder S-matrix, unpacked once per scan (k_rows_unpack);
 //   k_rows_window  per (raster row, Lp consecutive probes): psi on (x, ky), the row transforms, the
 //                  intensities, folded over +-kx and +-ky (the annular bins depend on |kx|, |ky|)
 //                  into shared memory, then the bins -- or the full pattern.
@@ -19,6 +21,8 @@
 // Measured (40 000 probes of the 1024^2 carbon cell, 129 beams, 64-pixel windows): 5.03 ms with the
 // blocks of scan_gemm.cuh, 1.51 ms here (k_rows_sum 0.61, k_rows_window 0.84); 32 x 32 probes of the
 // 2048^2 cell (529 beams, 128-pixel windows) 2.68 -> 0.76 ms; 16 x 16 probes of a 256^2 cell 68 -> 33 us.
+// 33 x 31 probes of a 512^2 cell from value + remainder storage (213 beams): 382 us on the tensor cores,
+// 110 us here, nearer to 64 bits (2.3e-6 against 4.9e-6 off).
 // Bound: k_rows_sum by the load/store pipe (67 % busy; its S reads hit the L2, 1.9 GB of them),
 // k_rows_window by the same pipe (60 %) and dependent latency at 16 warps per SM (issue slots 49 %);
 // leaving out the products saves 32 % of its time, the loads of the planes 20 %, the transforms 12 %,
@@ -110,14 +114,15 @@ __global__ void __launch_bounds__(RowsSumCfg<NWY>::BLOCK, 3) k_rows_sum(const __
     __syncthreads();
     const int ytop = geo[0], yn = geo[1];
     const int col = 2 * (tid % C::PAIRS);
-    const int x = (a.rows_g0 + blockIdx.x * XC + col) & (a.nx_s - 1);  // even: the pair is one aligned load
-    const size_t npix = (size_t)a.ny_s * a.nx_s;
+    // even: the pair is one aligned load
+    const int x = (a.rows_g0 + blockIdx.x * XC + col - a.rows_x0) & (a.nx_s - 1);
+    const size_t npix = (size_t)a.rows_ry * a.rows_pitch;
     for (int yv = tid / C::PAIRS; yv < yn; yv += C::YSTEP) {
         bool any = false;
 #pragma unroll
         for (int r = 0; r < R; ++r) any = any || (unsigned)(yv - wy0[r]) < (unsigned)NWY;
         if (!any) continue;  // between the windows of rows far apart
-        const float2 *sp = a.S + (size_t)((ytop + yv) & (a.ny_s - 1)) * a.nx_s + x;
+        const float2 *sp = a.rows_src + (size_t)((ytop + yv - a.rows_y0) & (a.ny_s - 1)) * a.rows_pitch + x;
 #pragma unroll 1
         for (int sg = 0; sg < 2; ++sg) {
             // T = sum_b Re S_b c_b + i sum_b Im S_b c_b, both as packed FMAs, combined at the end (the
@@ -447,7 +452,7 @@ static cudaError_t rows_launch(const ScanArgs &args, cudaStream_t s) {
     using A = RowsSumCfg<NWY>;
     using B = RowsWinCfg<NWX, NWY>;
     ScanArgs a = args;
-    if (reinterpret_cast<uintptr_t>(a.S) & 15) return cudaErrorMisalignedAddress;  // pixel pairs are read as one load
+    if (reinterpret_cast<uintptr_t>(a.rows_src) & 15) return cudaErrorMisalignedAddress;  // pixel pairs are read as one load
     const int kp = rows_kp(a.rows_m);
     const size_t sa = A::smem(a.rows_maxn), sb = B::smem(a.rows_lp, rows_mp(a.rows_m), a.n_fold16);
     void (*sum)(const ScanArgs) = k_rows_sum<NWY>;

@@ -13,8 +13,8 @@ from paper_1702_01904_gb300.runtime import PrismSimulation  # noqa: E402
 pytestmark = pytest.mark.gpu
 
 
-def plan(n, cell, f, f_y, alpha, seed):
-    sim = PrismSimulation(P.make_grid(n, n, 1, cell, cell, 2.0, 300.0, f, 2, 0.5, alpha, f_y=f_y))
+def plan(n, cell, f, f_y, alpha, seed, precision=P.PRISM_PRECISION_FP32):
+    sim = PrismSimulation(P.make_grid(n, n, 1, cell, cell, 2.0, 300.0, f, 2, 0.5, alpha, f_y=f_y, precision=precision))
     i = sim.info
     g = torch.Generator(device="cuda").manual_seed(seed)
     S = torch.randn((i.n_beams, i.ny_s, i.nx_s, 2), generator=g, device="cuda")
@@ -22,10 +22,11 @@ def plan(n, cell, f, f_y, alpha, seed):
     return sim
 
 
-def close(got, ref, beams):
+def close(got, ref, beams, product=0.0):
     # both sum the same products in FP32 in another order: at most one rounding of 2^-24 per beam and per
     # butterfly stage (two transforms of up to 7 stages, and the combinations), twice that for intensities
-    tol = 2.0 * (beams + 24) * 2.0 ** -24
+    # (product: a relative error of every product besides, which add up like the random values do)
+    tol = 2.0 * (beams + 24) * 2.0 ** -24 + 2.0 * product * beams ** 0.5
     err = np.linalg.norm(got.astype(np.float64) - ref) / np.linalg.norm(ref)
     assert err <= tol, (err, tol)
 
@@ -102,4 +103,21 @@ def test_rows_partition_and_repeat_bitwise():
             k = min(rows, 23 - r)
             part = sim.scan(probe, x0[r * 40:(r + k) * 40], y0[r * 40:(r + k) * 40], det, px=40, py=k).cpu().numpy()
             assert np.array_equal(part, whole[r * 40:(r + k) * 40])
+    sim.close()
+
+
+@pytest.mark.parametrize("n,cell,f,alpha", [(64, 8.0, 2, 20.0), (256, 16.0, 4, 20.0), (256, 12.5, 2, 28.0)])
+@pytest.mark.parametrize("kind,px,py,step", [("wrap", 33, 9, 0.21), ("serpentine", 9, 30, 0.05), ("skew", 40, 17, 0.4),
+                                             ("plain", 4, 4, 0.3)])
+def test_rows_of_value_and_remainder_storage(n, cell, f, alpha, kind, px, py, step):
+    # the unpacked S-matrix against the tensor-core scan of the position list, whose products carry 22-bit
+    # coefficients and leave out remainder x remainder (2^-22 each, with the 22-bit values at most 2^-20 in all)
+    sim = plan(n, cell, f, 0, alpha, 8, P.PRISM_PRECISION_FP16X2)
+    x0, y0 = raster(kind, cell, px, py, step)
+    probe, det = P.make_probe(20.0, 30.0), P.make_detector(0.0, 2.0, 40)
+    got = sim.scan(probe, x0, y0, det, px=px, py=py).cpu().numpy()
+    ref = sim.scan(probe, x0, y0, det).cpu().numpy()
+    close(got, ref, sim.info.n_beams, 2.0 ** -20)
+    cb = sim.scan_cbed(probe, x0, y0, px=px, py=py).cpu().numpy()
+    close(cb, sim.scan_cbed(probe, x0, y0).cpu().numpy(), sim.info.n_beams, 2.0 ** -20)
     sim.close()
