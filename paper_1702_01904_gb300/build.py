@@ -22,7 +22,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libprism.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 HEADERS = [os.path.join(CSRC, h) for h in ("fft.cuh", "params.h", "internal.h", "tc.cuh", "scan_common.cuh", "pass_kernels.cuh",
-                                           "tune_shapes.cuh", "tune_pass.cuh", "scan_gemm.cuh", "scan_tc.cuh", "scan_rows.cuh",
+                                           "tune_shapes.cuh", "tune_pass.cuh", "scan_gemm.cuh", "scan_tc.cuh", "scan_rows.cuh", "launch.cuh",
                                            "pass_default.cuh")] + \
     [os.path.join(INCLUDE, "prism.h")]
 CUDA_UNITS = ["kernels_build.cu", "kernels_pass_512.cu", "kernels_pass_1024.cu", "kernels_pass_2048.cu", "kernels_tune.cu",

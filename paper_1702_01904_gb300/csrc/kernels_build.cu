@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "fft.cuh"
+#include "launch.cuh"
 #include "params.h"
 #include "pass_default.cuh"
 #include "pass_kernels.cuh"
@@ -18,6 +19,8 @@ namespace prism {
 // exact while |p| < 2^23).
 __global__ void __launch_bounds__(256) k_transmission(const float4 *__restrict__ V, float4 *__restrict__ t,
                                                       size_t n4, float sig_hi, float sig_lo) {
+    next_may_start();
+    after_previous();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
         const float4 v = V[i];
         float vv[4] = {v.x, v.y, v.z, v.w};
@@ -52,6 +55,8 @@ __global__ void __launch_bounds__(256) k_plane(const float2 *__restrict__ T0, fl
     // or no pruning), so rows go as 16-byte pixel pairs
     const bool pairs = (f & 1) == 0 && (kx_half & 1) == 0 && (nx & 1) == 0;
     const int npairs = kx_half > 0 ? kx_half : nx / 2;  // kh/2 low + kh/2 high pairs, or all
+    next_may_start();
+    after_previous();
     for (int row = blockIdx.x; row < nb * ny; row += gridDim.x) {
         const int b = row / ny, y = row - b * ny;
         const int m = __ldg(beam_mn + 2 * (beam0 + b)), n = __ldg(beam_mn + 2 * (beam0 + b) + 1);
@@ -88,8 +93,7 @@ cudaError_t launch_plane(const float2 *T0, float2 *wave, const int *beam_mn, int
     if (nb <= 0) return cudaSuccess;
     if ((nx & (nx - 1)) || (ny & (ny - 1))) return cudaErrorInvalidValue;  // the masks need powers of two
     const int rows = nb * ny;
-    k_plane<<<rows < 152 * 8 ? rows : 152 * 8, 256, 0, s>>>(T0, wave, beam_mn, beam0, nb, nx, ny, f, f_y, kx_half);
-    return cudaGetLastError();
+    return launch_chained(k_plane, rows < 152 * 8 ? rows : 152 * 8, 256, 0, s, T0, wave, beam_mn, beam0, nb, nx, ny, f, f_y, kx_half);
 }
 
 cudaError_t launch_transmission(const float *V, float2 *t, size_t n, double sigma_cycles, cudaStream_t s) {
@@ -98,9 +102,8 @@ cudaError_t launch_transmission(const float *V, float2 *t, size_t n, double sigm
     size_t blocks = (n4 + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
     const float hi = (float)sigma_cycles, lo = (float)(sigma_cycles - (double)hi);
-    k_transmission<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4 *>(V),
-                                                     reinterpret_cast<float4 *>(t), n4, hi, lo);
-    return cudaGetLastError();
+    return launch_chained(k_transmission, (unsigned)blocks, 256, 0, s, reinterpret_cast<const float4 *>(V),
+                          reinterpret_cast<float4 *>(t), n4, hi, lo);
 }
 
 // ------------------------------------------------------------------ default launch shapes
@@ -179,6 +182,8 @@ void fft_split(int n, int *n1, int *n2) {
 // ------------------------------------------------------------------ probe shift phases
 // shift_x[b][k] = exp(-2 pi i (k/cell_x) x0_b); the phase is reduced in FP64 before FP32 sincos.
 __global__ void k_shift(const __grid_constant__ ShiftArgs a) {
+    next_may_start();
+    after_previous();
     const int b = blockIdx.y;
     const double x0 = a.x0[b], y0 = a.y0[b];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.nx + a.ny; i += gridDim.x * blockDim.x) {
@@ -201,14 +206,15 @@ __global__ void k_shift(const __grid_constant__ ShiftArgs a) {
 cudaError_t launch_shift(const ShiftArgs &a, cudaStream_t s) {
     if (a.batch <= 0) return cudaSuccess;
     const dim3 grid((a.nx + a.ny + 255) / 256, a.batch);
-    k_shift<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_shift, grid, 256, 0, s, a);
 }
 
 // ------------------------------------------------------------------ detector bins
 // out[b][k] = scale * sum_{pixels in bin k} inten[b][pixel]: one warp per bin, FP64 lane sums in a
 // fixed order and a fixed xor-shuffle tree (bitwise reproducible).
 __global__ void __launch_bounds__(256) k_bins(const __grid_constant__ BinArgs a) {
+    next_may_start();
+    after_previous();
     const int b = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float *img = a.inten + (size_t)b * a.npix;
@@ -225,8 +231,7 @@ __global__ void __launch_bounds__(256) k_bins(const __grid_constant__ BinArgs a)
 
 cudaError_t launch_bins(const BinArgs &a, cudaStream_t s) {
     if (a.batch <= 0) return cudaSuccess;
-    k_bins<<<a.batch, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_bins, a.batch, 256, 0, s, a);
 }
 
 }  // namespace prism

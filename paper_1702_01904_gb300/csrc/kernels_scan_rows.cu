@@ -22,6 +22,8 @@ __global__ void __launch_bounds__(256) k_rows_unpack(const __grid_constant__ Sca
     const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int x0 = blockIdx.x * 32, y = blockIdx.y, b0 = blockIdx.z * 32;
     const int b = b0 + lane;
+    next_may_start();
+    after_previous();
     const uint32_t *src = reinterpret_cast<const uint32_t *>(a.S16) + (size_t)((a.rows_y0 + y) & (a.ny_s - 1)) * a.nx_s * a.kp;
     if (b < a.n_beams) {
         const float sc = a.beam_scale[b];
@@ -52,8 +54,7 @@ cudaError_t launch_scan_rows(int nwx, int nwy, const ScanArgs &a, cudaStream_t s
     if (!a.rows_w || !a.rows_src || a.rows_lp <= 0 || a.rows_chunk <= 0 || a.scan_px <= 0 || a.scan_py <= 0) return cudaErrorInvalidValue;
     if (a.rows_unpack) {
         const dim3 grid((a.rows_pitch + 31) / 32, a.rows_ry, (a.n_beams + 31) / 32);
-        k_rows_unpack<<<grid, 256, 0, s>>>(a, const_cast<float2 *>(a.rows_src));
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_chained(k_rows_unpack, grid, 256, 0, s, a, const_cast<float2 *>(a.rows_src));
         if (e != cudaSuccess) return e;
     }
 #define PRISM_ROWS_LAUNCH(x, y) \

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "fft.cuh"
+#include "launch.cuh"
 #include "params.h"
 #include "tc.cuh"  // mbarrier and TMA helpers
 
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(THR) k_row(const __grid_constant__ RowArgs a) 
     constexpr unsigned long long ZIN = BL && MODE != ROW_PLANE ? band_zero_mask<Inv, NX>(true) : 0ull;
     extern __shared__ float2 smem[];
     __shared__ __align__(8) uint64_t rbar[C::SLOTS];  // TM: a slot's next row has landed
+    next_may_start();
     uint32_t rphase = 0;
     const int slot = threadIdx.x / T, t = threadIdx.x % T;
     if constexpr (C::TMA) {
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(THR) k_row(const __grid_constant__ RowArgs a) 
             tc::bulk_load(stg + NX / 4, w + 3 * NX / 4, (uint32_t)(NX / 4 * sizeof(float2)), &rbar[slot]);
         }
     };
+    after_previous();
     if constexpr (C::TMA) bulk(row0);
     if constexpr (MODE != ROW_PLANE && C::STAGE) stage(row0);
     for (int it = 0; it < iters; ++it) {
@@ -326,8 +329,7 @@ static cudaError_t row_go_bl(const RowArgs &a, cudaStream_t s) {
     cudaError_t e = persistent_grid(k_row<NX, MODE, THR, STG, BL, TM, RV>, C::THREADS, C::SMEM, (a.n_rows + C::SLOTS - 1) / C::SLOTS,
                                     &grid, C::PERSIST);
     if (e != cudaSuccess) return e;
-    k_row<NX, MODE, THR, STG, BL, TM, RV><<<grid, C::THREADS, C::SMEM, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_row<NX, MODE, THR, STG, BL, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
 }
 
 // TM: bulk staging where it applies (the compile-time band, one slot per warp, rows read from the
@@ -403,6 +405,7 @@ __global__ void __launch_bounds__(ColCfg<NY, WC, STG, MB, TM>::THREADS, ColCfg<N
     float2 *smem = smem_c;
     __shared__ __align__(8) uint64_t tbar;  // TMA staging: the tile's boxes have landed
     __shared__ int s_next;                  // TMA staging with a tile counter: the next tile
+    next_may_start();
     uint32_t tphase = 0;
     if constexpr (C::TMA) {
         if (threadIdx.x == 0) {
@@ -487,6 +490,7 @@ __global__ void __launch_bounds__(ColCfg<NY, WC, STG, MB, TM>::THREADS, ColCfg<N
             if constexpr (cls != BAND_OUT) pyr[r] = __ldg(a.prop_y + Fwd::out_elem(r, t));
         });
     }
+    after_previous();
     // TMA-staged shapes given a tile counter take their tiles from it, each one tile ahead (the
     // tile the prefetch loads), instead of by a fixed stride: the CTAs sharing an SM are not issued
     // equally, and with fixed shares the favoured ones finished early (per-CTA times of 170 to
@@ -673,14 +677,12 @@ static cudaError_t col_go(const ColArgs &a, cudaStream_t s) {
             if (a.band4) {
                 e = persistent_grid(k_col<NY, MODE, WC, STG, MB, true, TM, RV>, C::THREADS, C::SMEM, work, &grid, C::PERSIST);
                 if (e != cudaSuccess) return e;
-                k_col<NY, MODE, WC, STG, MB, true, TM, RV><<<grid, C::THREADS, C::SMEM, s>>>(a);
-                return cudaGetLastError();
+                return launch_chained(k_col<NY, MODE, WC, STG, MB, true, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
             }
         }
         e = persistent_grid(k_col<NY, MODE, WC, STG, MB, false, TM, RV>, C::THREADS, C::SMEM, work, &grid, C::PERSIST);
         if (e != cudaSuccess) return e;
-        k_col<NY, MODE, WC, STG, MB, false, TM, RV><<<grid, C::THREADS, C::SMEM, s>>>(a);
-        return cudaGetLastError();
+        return launch_chained(k_col<NY, MODE, WC, STG, MB, false, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
     }
 }
 

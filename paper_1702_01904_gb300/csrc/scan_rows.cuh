@@ -33,6 +33,7 @@
 #include <algorithm>
 
 #include "fft.cuh"
+#include "launch.cuh"
 #include "params.h"
 #include "scan_common.cuh"
 
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(RowsSumCfg<NWY>::BLOCK, 3) k_rows_sum(const __
     int *beam = reinterpret_cast<int *>(coef + (np + nm) * R);
     __shared__ int wy0[R];   // window row origins relative to the first union row (out of reach: no such row)
     __shared__ int geo[2];   // first union row, union rows
+    next_may_start();
     for (int i = tid; i < np + nm; i += BLOCK) beam[i] = __ldg(a.m_beam + (i < np ? pb + i : mb + i - np));
     for (int i = tid; i < (np + nm) * R; i += BLOCK) {
         const int k = i / R, r = i - k * R;
@@ -112,6 +114,7 @@ __global__ void __launch_bounds__(RowsSumCfg<NWY>::BLOCK, 3) k_rows_sum(const __
         }
     }
     __syncthreads();
+    after_previous();
     const int ytop = geo[0], yn = geo[1];
     const int col = 2 * (tid % C::PAIRS);
     // even: the pair is one aligned load
@@ -248,6 +251,7 @@ __global__ void __launch_bounds__(RowsWinCfg<NWX, NWY>::BLOCK, RowsWinCfg<NWX, N
     float2 *win = reinterpret_cast<float2 *>(cs + LP * MP) + (size_t)warp * 2 * C::padded(LP) * PITCH;  // [2][probe][PITCH]
     const int row1 = C::padded(LP) * PITCH;  // to the second row of a pair
     float *fold = reinterpret_cast<float *>(reinterpret_cast<float2 *>(cs + LP * MP) + (size_t)C::WARPS * 2 * C::padded(LP) * PITCH);  // [LP][FY][FX]
+    next_may_start();
     // the bins' offsets and lists, read after the windows
     uint16_t *lists = reinterpret_cast<uint16_t *>(fold + ((LP * FX * FY + 3) & ~3));
     for (int i = tid; i < a.n_fold16 / 8; i += BLOCK) cp_async16(lists + 8 * i, a.fold16 + 8 * i);
@@ -278,6 +282,7 @@ __global__ void __launch_bounds__(RowsWinCfg<NWX, NWY>::BLOCK, RowsWinCfg<NWX, N
         }
     }
     __syncthreads();
+    after_previous();
     const int xf = geo[0], vc = geo[1];
     const size_t rstride = (size_t)npl * a.rows_cols;  // W: one ky
     const float2 *wrow = a.rows_w + (size_t)row * NWY * rstride;
@@ -467,10 +472,8 @@ static cudaError_t rows_launch(const ScanArgs &args, cudaStream_t s) {
         a.rows_0 = r0;
         a.rows_n = std::min(a.rows_chunk, a.scan_py - r0);
         const dim3 ga(a.rows_cols / A::XC, a.rows_m + 1, (a.rows_n + ROWS_R - 1) / ROWS_R);
-        sum<<<ga, A::BLOCK, sa, s>>>(a);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        win<<<a.rows_n * ngc, B::BLOCK, sb, s>>>(a);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_chained(sum, ga, A::BLOCK, sa, s, a)) != cudaSuccess) return e;
+        if ((e = launch_chained(win, a.rows_n * ngc, B::BLOCK, sb, s, a)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
