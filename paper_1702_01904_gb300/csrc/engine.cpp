@@ -250,21 +250,18 @@ static int build_grid_tables(const prism_grid *g, GridTables &T) {
     T.aa_kmax.assign(T.nx, -1);
     for (int kx = 0; kx < T.nx; ++kx) {
         const double qx = (double)signed_index(kx, T.nx) / g->cell_x;
-        int kmax = -1;
-        for (int ky = 0; ky < T.ny; ++ky) {
-            const int ks = signed_index(ky, T.ny);
+        const auto in = [&](int ks) {
             const double qy = (double)ks / g->cell_y;
-            const bool in = qx * qx + qy * qy < qaa2;
-            if (in) kmax = std::max(kmax, std::abs(ks));
+            return qx * qx + qy * qy < qaa2;
+        };
+        // |q| grows with |ky| (in floating point too: every operation is monotone) and is the same for +-ky,
+        // so the mask is the interval |ky| <= kmax: bisect for its end; ky = -ny/2 has no mirror
+        int lo = -1, hi = T.ny / 2;  // in(lo) or lo = -1, not in(hi) or hi = ny/2
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) / 2;
+            (in(mid) ? lo : hi) = mid;
         }
-        // the mask must be the symmetric interval |ky| <= kmax
-        for (int ky = 0; ky < T.ny; ++ky) {
-            const int ks = signed_index(ky, T.ny);
-            const double qy = (double)ks / g->cell_y;
-            const bool in = qx * qx + qy * qy < qaa2;
-            if (in != (std::abs(ks) <= kmax)) return fail(PRISM_ERR_INVALID, "anti-aliasing mask is not a symmetric interval");
-        }
-        T.aa_kmax[kx] = kmax;
+        T.aa_kmax[kx] = in(-T.ny / 2) ? T.ny / 2 : lo;
     }
     // columns that pass the aperture: |kx| <= K, a symmetric interval (else no pruning)
     int K = -1;
@@ -1276,15 +1273,46 @@ extern "C" int prism_scan_run_accumulate(prism_plan *P, const prism_probe *probe
 }
 
 // ------------------------------------------------------------------ multislice baseline
+// The pixels ky * nx + kx (FFT order, ascending) inside the probe's aperture and A(q - q_t) exp(-i chi(q -
+// q_t)) there; every other pixel is zero.  Only the pixels about the aperture's centre are looked at: beyond
+// alpha / lambda (and a pixel's margin) of it, lambda |q - q_t| > alpha.
+static void probe_entries(const prism_grid &g, double lam, const prism_probe *probe, const Tilt &tl, std::vector<int> &idx,
+                          std::vector<float2> &val) {
+    const double alpha = probe->alpha_mrad * 1e-3, reach = alpha / lam * (1.0 + 1e-6);
+    const auto range = [&](double centre, double cell, int n, int *lo, int *hi) {
+        *lo = (int)std::max(-n / 2.0, std::floor((centre - reach) * cell) - 1.0);
+        *hi = (int)std::min(n / 2.0 - 1.0, std::ceil((centre + reach) * cell) + 1.0);
+    };
+    int x0, x1, y0, y1;
+    range(tl.qtx, g.cell_x, g.nx, &x0, &x1);
+    range(tl.qty, g.cell_y, g.ny, &y0, &y1);
+    const auto line = [&](int ks) {
+        const double qy = (double)ks / g.cell_y;
+        const int ky = ks < 0 ? ks + g.ny : ks;
+        const auto pixel = [&](int xs) {
+            const double qx = (double)xs / g.cell_x;
+            const double dqx = qx - tl.qtx;
+            const double dqy = qy - tl.qty;
+            if (inside_aperture(dqx, dqy, lam, alpha)) {
+                idx.push_back(ky * g.nx + (xs < 0 ? xs + g.nx : xs));
+                val.push_back(phase_cycles(chi_cycles(dqx * dqx + dqy * dqy, lam, probe->c1, probe->c3)));
+            }
+        };
+        for (int xs = std::max(x0, 0); xs <= x1; ++xs) pixel(xs);
+        for (int xs = x0; xs <= std::min(x1, -1); ++xs) pixel(xs);
+    };
+    for (int ks = std::max(y0, 0); ks <= y1; ++ks) line(ks);
+    for (int ks = y0; ks <= std::min(y1, -1); ++ks) line(ks);
+}
+
 // The row passes may skip the columns the anti-aliasing aperture zeroes (|kx| >= kx_half) only if
 // the initial probe is zero there too: a probe aperture wider than the anti-aliasing aperture keeps
 // every column (returns 0).
-static int probe_kx_half(int kx_half, const std::vector<float2> &pbase, int nx, int ny) {
-    for (int ky = 0; ky < ny && kx_half; ++ky)
-        for (int kx = kx_half; kx <= nx - kx_half; ++kx) {
-            const float2 v = pbase[(size_t)ky * nx + kx];
-            if (v.x != 0.f || v.y != 0.f) return 0;
-        }
+static int probe_kx_half(int kx_half, const std::vector<int> &idx, int nx) {
+    for (const int i : idx) {
+        const int kx = i % nx;
+        if (kx_half && kx >= kx_half && kx <= nx - kx_half) return 0;
+    }
     return kx_half;
 }
 
@@ -1308,25 +1336,11 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
     const size_t px = (size_t)nx * ny;
     // probe A(q - q_t) exp(-i chi(q - q_t)) on the full grid, sum |Psi0|^2 = aperture pixel count
     const Tilt tl = tilt_terms(probe, T.lam, T.dz);
-    std::vector<float2> pbase(px);
-    double count = 0;
-    for (int ky = 0; ky < ny; ++ky) {
-        const double qy = (double)signed_index(ky, ny) / g.cell_y;
-        for (int kx = 0; kx < nx; ++kx) {
-            const double qx = (double)signed_index(kx, nx) / g.cell_x;
-            const double dqx = qx - tl.qtx;
-            const double dqy = qy - tl.qty;
-            if (inside_aperture(dqx, dqy, T.lam, probe->alpha_mrad * 1e-3)) {
-                pbase[(size_t)ky * nx + kx] = phase_cycles(chi_cycles(dqx * dqx + dqy * dqy, T.lam, probe->c1, probe->c3));
-                count += 1.0;
-            } else {
-                pbase[(size_t)ky * nx + kx] = make_float2(0.f, 0.f);
-            }
-        }
-    }
-    const int kx_half = probe_kx_half(T.kx_half, pbase, nx, ny);
-    std::vector<int> off, idx;
-    detector_csr(nx, ny, g.cell_x, g.cell_y, 1, 1, T.lam, det, off, idx);
+    std::vector<int> pidx;
+    std::vector<float2> pval;
+    probe_entries(g, T.lam, probe, tl, pidx, pval);
+    const double count = (double)pidx.size();
+    const int kx_half = probe_kx_half(T.kx_half, pidx, nx);
     if (scratch_bytes == 0) scratch_bytes = (size_t)1 << 30;
     const int Pb = (int)std::max<long long>(1, std::min<long long>(Pn, (long long)(scratch_bytes / (px * 8))));
     const Tw64 tw = make_tw64();
@@ -1354,9 +1368,28 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
     if ((rc = A.upload(&twr_i, T.twr_i))) return done(rc);
     if ((rc = A.upload(&twc_f, T.twc_f))) return done(rc);
     if ((rc = A.upload(&twc_i, T.twc_i))) return done(rc);
-    if ((rc = A.upload(&pb, pbase))) return done(rc);
-    if ((rc = A.upload(&d_off, off))) return done(rc);
-    if ((rc = A.upload(&d_idx, idx))) return done(rc);
+    int *p_idx;
+    float2 *p_val;
+    if ((rc = A.upload(&p_idx, pidx))) return done(rc);
+    if ((rc = A.upload(&p_val, pval))) return done(rc);
+    if ((rc = A.alloc((void **)&pb, px * sizeof(float2)))) return done(rc);
+    BinListArgs bl;
+    bl.nx = nx;
+    bl.ny = ny;
+    bl.nbins = det->nbins;
+    bl.cell_x = g.cell_x;
+    bl.cell_y = g.cell_y;
+    bl.lam = T.lam;
+    bl.start = det->start_mrad;
+    bl.step = det->step_mrad;
+    if ((rc = A.alloc((void **)&bl.map, (size_t)(ny / 2 + 1) * (nx / 2 + 1) * sizeof(uint16_t)))) return done(rc);
+    if ((rc = A.alloc((void **)&bl.rows, (size_t)(ny / 2 + 1) * det->nbins * sizeof(int)))) return done(rc);
+    if ((rc = A.alloc((void **)&bl.base, (size_t)ny * det->nbins * sizeof(int)))) return done(rc);
+    if ((rc = A.alloc((void **)&bl.total, (size_t)det->nbins * sizeof(int)))) return done(rc);
+    if ((rc = A.alloc((void **)&d_off, (size_t)(det->nbins + 1) * sizeof(int)))) return done(rc);
+    if ((rc = A.alloc((void **)&d_idx, px * sizeof(int)))) return done(rc);
+    bl.off = d_off;
+    bl.idx = d_idx;
     if ((rc = A.alloc((void **)&pos, (size_t)Pn * 2 * sizeof(double)))) return done(rc);
     // the column passes between slices as in a plan's build: from 256^2 to 1024^2 the TMA-staged shapes
     // where they are the default (tiles loaded and stored by TMA through tensor maps of this call's wave
@@ -1390,6 +1423,8 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
         if (err != cudaSuccess) return fail(PRISM_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(err));
         return PRISM_OK;
     };
+    if ((rc = check(launch_probe_base({p_idx, p_val, pb, (int)pidx.size()}, px, st), "probe base"))) return done(rc);
+    if ((rc = check(launch_bin_lists(bl, st), "detector lists"))) return done(rc);
     if ((rc = check(launch_transmission(V_dev, t, (size_t)g.n_slices * px, T.sigma / (2.0 * PI), st), "transmission"))) return done(rc);
     for (long long p0 = 0; p0 < Pn; p0 += Pb) {
         const int nb = (int)std::min<long long>(Pb, Pn - p0);
@@ -1658,20 +1693,12 @@ int internal_multislice_tables(const prism_grid *grid, const prism_probe *probe,
     const size_t px = (size_t)g.nx * g.ny;
     const Tilt tl = tilt_terms(probe, T.lam, T.dz);
     M.pbase.assign(px, make_float2(0.f, 0.f));
-    M.count = 0;
-    for (int ky = 0; ky < g.ny; ++ky) {
-        const double qy = (double)signed_index(ky, g.ny) / g.cell_y;
-        for (int kx = 0; kx < g.nx; ++kx) {
-            const double qx = (double)signed_index(kx, g.nx) / g.cell_x;
-            const double dqx = qx - tl.qtx;
-            const double dqy = qy - tl.qty;
-            if (inside_aperture(dqx, dqy, T.lam, probe->alpha_mrad * 1e-3)) {
-                M.pbase[(size_t)ky * g.nx + kx] = phase_cycles(chi_cycles(dqx * dqx + dqy * dqy, T.lam, probe->c1, probe->c3));
-                M.count += 1.0;
-            }
-        }
-    }
-    M.kx_half = probe_kx_half(T.kx_half, M.pbase, g.nx, g.ny);
+    std::vector<int> pidx;
+    std::vector<float2> pval;
+    probe_entries(g, T.lam, probe, tl, pidx, pval);
+    for (size_t i = 0; i < pidx.size(); ++i) M.pbase[pidx[i]] = pval[i];
+    M.count = (double)pidx.size();
+    M.kx_half = probe_kx_half(T.kx_half, pidx, g.nx);
     M.band4 = T.band4;
     detector_csr(g.nx, g.ny, g.cell_x, g.cell_y, 1, 1, T.lam, det, M.bin_off, M.bin_idx);
     const long long Pn = (long long)sc->px * sc->py;

@@ -209,16 +209,153 @@ cudaError_t launch_shift(const ShiftArgs &a, cudaStream_t s) {
     return launch_chained(k_shift, grid, 256, 0, s, a);
 }
 
+// ------------------------------------------------------------------ probe base and detector lists
+__global__ void k_probe_base(const __grid_constant__ ProbeBaseArgs a) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) a.base[a.idx[i]] = a.val[i];
+}
+
+cudaError_t launch_probe_base(const ProbeBaseArgs &a, size_t npix, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(a.base, 0, npix * sizeof(float2), s);
+    if (e != cudaSuccess || a.n <= 0) return e;
+    k_probe_base<<<(a.n + 255) / 256 < 64 ? (a.n + 255) / 256 : 64, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+// The lists that detector_csr (engine.cpp) makes, without the 1 M-pixel loop and its 4 MB pageable copy on
+// the host, which held back the stream (at 1024^2, 12 ms of host work per call, 2 ms of it with the GPU
+// idle).  The bin of a pixel takes the same FP64 operations in the same order, none contracted.  Along a
+// row the bin grows with |kx|, so the pixels of a bin are one run on the side kx >= 0 and one on the other:
+// a pixel's rank in its list follows from the runs' starts.  All counts are integers: any order of the
+// atomics gives the same lists.
+__global__ void __launch_bounds__(256) k_bin_rows(const __grid_constant__ BinListArgs a) {
+    extern __shared__ int hist[];
+    const int j = blockIdx.x, hx = a.nx / 2;
+    next_may_start();
+    for (int k = threadIdx.x; k < a.nbins; k += 256) hist[k] = 0;
+    __syncthreads();
+    after_previous();
+    const double qy = __ddiv_rn((double)j, a.cell_y), c = __dmul_rn(1000.0, a.lam);
+    for (int i = threadIdx.x; i <= hx; i += 256) {
+        const double qx = __ddiv_rn((double)i, a.cell_x);
+        const double theta = __dmul_rn(c, __dsqrt_rn(__dadd_rn(__dmul_rn(qx, qx), __dmul_rn(qy, qy))));
+        const double bf = floor(__ddiv_rn(__dadd_rn(theta, -a.start), a.step));
+        const int b = bf >= 0.0 && bf < (double)a.nbins ? (int)bf : -1;
+        a.map[(size_t)j * (hx + 1) + i] = (uint16_t)b;
+        if (b >= 0) atomicAdd(&hist[b], i == 0 || i == hx ? 1 : 2);  // kx and -kx; 0 and -nx/2 stand alone
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < a.nbins; k += 256) a.rows[(size_t)j * a.nbins + k] = hist[k];
+}
+
+// pixels of the rows before, per bin: one warp per bin, each lane a run of rows
+__global__ void __launch_bounds__(128) k_bin_base(const __grid_constant__ BinListArgs a) {
+    const int k = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    next_may_start();
+    after_previous();
+    if (k >= a.nbins) return;
+    const int per = (a.ny + 31) / 32, y0 = lane * per, y1 = min(a.ny, y0 + per);
+    auto row = [&](int y) { return __ldcg(a.rows + (size_t)(y <= a.ny / 2 ? y : a.ny - y) * a.nbins + k); };
+    int sum = 0;
+#pragma unroll 8
+    for (int y = y0; y < y1; ++y) sum += row(y);
+    int before = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += v;
+    }
+    if (lane == 31) a.total[k] = before;
+    before -= sum;
+#pragma unroll 8
+    for (int y = y0; y < y1; ++y) {
+        a.base[(size_t)y * a.nbins + k] = before;
+        before += row(y);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_bin_fill(const __grid_constant__ BinListArgs a) {
+    extern __shared__ int sm_bins[];
+    int *at = sm_bins, *pos = at + a.nbins, *neg = pos + a.nbins;  // list position of the row, first kx of either run
+    int *npos = neg + a.nbins;                                     // pixels of the run kx >= 0
+    __shared__ int part[256];
+    const int y = blockIdx.x, hx = a.nx / 2, tid = threadIdx.x;
+    next_may_start();
+    for (int k = tid; k < a.nbins; k += 256) {
+        pos[k] = neg[k] = 1 << 30;
+        npos[k] = 0;
+    }
+    after_previous();
+    // list offsets: exclusive sums of the totals, a run of bins per thread
+    const int per = (a.nbins + 255) / 256, k0 = min(a.nbins, tid * per), k1 = min(a.nbins, k0 + per);
+    int sum = 0;
+    for (int k = k0; k < k1; ++k) sum += __ldcg(a.total + k);
+    part[tid] = sum;
+    __syncthreads();
+    if (tid < 32) {
+        int s = 0;
+        for (int i = 0; i < 8; ++i) s += part[tid * 8 + i];
+        int inc = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (tid >= o) inc += v;
+        }
+        inc -= s;
+        for (int i = 0; i < 8; ++i) {
+            const int v = part[tid * 8 + i];
+            part[tid * 8 + i] = inc;
+            inc += v;
+        }
+    }
+    __syncthreads();
+    int o = part[tid];
+    for (int k = k0; k < k1; ++k) {
+        if (y == 0) a.off[k] = o;
+        at[k] = o + __ldcg(a.base + (size_t)y * a.nbins + k);
+        o += __ldcg(a.total + k);
+    }
+    if (y == 0 && k1 == a.nbins && k0 < k1) a.off[a.nbins] = o;
+    const uint16_t *map = a.map + (size_t)(y <= a.ny / 2 ? y : a.ny - y) * (hx + 1);
+    for (int x = tid; x < a.nx; x += 256) {
+        const int b = __ldcg(map + (x <= hx ? x : a.nx - x));
+        if (b == 0xffff) continue;
+        if (x < hx) {
+            atomicMin(&pos[b], x);
+            atomicAdd(&npos[b], 1);
+        } else {
+            atomicMin(&neg[b], x);
+        }
+    }
+    __syncthreads();
+    for (int x = tid; x < a.nx; x += 256) {
+        const int b = __ldcg(map + (x <= hx ? x : a.nx - x));
+        if (b == 0xffff) continue;
+        a.idx[at[b] + (x < hx ? x - pos[b] : npos[b] + x - neg[b])] = y * a.nx + x;
+    }
+}
+
+cudaError_t launch_bin_lists(const BinListArgs &a, cudaStream_t s) {
+    // (nbins <= 4096: 64 KB of shared memory at most)
+    const size_t sr = (size_t)a.nbins * sizeof(int), sf = 4 * sr;
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_bin_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024)) != cudaSuccess) return e;
+    if ((e = launch_chained(k_bin_rows, a.ny / 2 + 1, 256, sr, s, a)) != cudaSuccess) return e;
+    if ((e = launch_chained(k_bin_base, (a.nbins + 3) / 4, 128, 0, s, a)) != cudaSuccess) return e;
+    return launch_chained(k_bin_fill, a.ny, 256, sf, s, a);
+}
+
 // ------------------------------------------------------------------ detector bins
 // out[b][k] = scale * sum_{pixels in bin k} inten[b][pixel]: one warp per bin, FP64 lane sums in a
-// fixed order and a fixed xor-shuffle tree (bitwise reproducible).
+// fixed order and a fixed xor-shuffle tree (bitwise reproducible).  A probe's bins are spread over
+// gridDim.y CTAs, so that a few probes still fill the SMs (100 probes of 1024^2 and 100 bins: 206 us with
+// one CTA per probe, 97 us spread).
 __global__ void __launch_bounds__(256) k_bins(const __grid_constant__ BinArgs a) {
     next_may_start();
     after_previous();
     const int b = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float *img = a.inten + (size_t)b * a.npix;
-    for (int k = warp; k < a.nbins; k += 8) {
+    for (int k = blockIdx.y * 8 + warp; k < a.nbins; k += 8 * gridDim.y) {
         double s = 0.0;
         const int e = a.bin_off[k + 1];
         for (int i = a.bin_off[k] + lane; i < e; i += 32) s += (double)__ldg(img + __ldg(a.bin_idx + i));
@@ -231,7 +368,8 @@ __global__ void __launch_bounds__(256) k_bins(const __grid_constant__ BinArgs a)
 
 cudaError_t launch_bins(const BinArgs &a, cudaStream_t s) {
     if (a.batch <= 0) return cudaSuccess;
-    return launch_chained(k_bins, a.batch, 256, 0, s, a);
+    const int want = (152 * 16 + a.batch - 1) / a.batch, most = (a.nbins + 7) / 8;
+    return launch_chained(k_bins, dim3(a.batch, want < most ? want : most), 256, 0, s, a);
 }
 
 }  // namespace prism

@@ -158,6 +158,26 @@ struct ShiftArgs {
     double cell_x, cell_y;
 };
 
+// The detector's pixel lists of a full grid, made on the device: CSR of the pixels ky * nx + kx (FFT order)
+// by bin = floor((1000 lambda |q| - start) / step), q = (kx / cell_x, ky / cell_y), each list in pixel order
+struct BinListArgs {
+    int nx, ny, nbins;
+    double cell_x, cell_y, lam, start, step;
+    uint16_t *map;             // [ny/2 + 1][nx/2 + 1] bin of (|ky|, |kx|), 0xffff: none
+    int *rows;                 // [ny/2 + 1][nbins] pixels of a row per bin
+    int *base;                 // [ny][nbins] pixels of the rows before
+    int *total;                // [nbins]
+    int *off;                  // [nbins + 1]
+    int *idx;                  // [nx * ny] at most
+};
+// the entries of a probe's aperture: base[idx[i]] = val[i], every other pixel zero
+struct ProbeBaseArgs {
+    const int *idx;
+    const float2 *val;
+    float2 *base;
+    int n;
+};
+
 struct BinArgs {
     const float *inten;        // [batch][npix]
     const int *bin_off;        // [nbins+1]
@@ -207,6 +227,8 @@ int scan_rows_lp(int nwx, int nwy, int m, int max_beams, int lists, int px, int 
 cudaError_t launch_scan_rows(int nwx, int nwy, const ScanArgs &a, cudaStream_t s);
 cudaError_t launch_shift(const ShiftArgs &a, cudaStream_t s);
 cudaError_t launch_bins(const BinArgs &a, cudaStream_t s);
+cudaError_t launch_bin_lists(const BinListArgs &a, cudaStream_t s);
+cudaError_t launch_probe_base(const ProbeBaseArgs &a, size_t npix, cudaStream_t s);
 cudaError_t launch_tc_selftest(float *out, int *status, cudaStream_t s);
 cudaError_t launch_wait_selftest(int *status, long long limit_cycles, int arrive, cudaStream_t s);
 // 16-bit mode (kernels_tc.cu)
