@@ -326,8 +326,8 @@ void prism_server_destroy(prism_server *server);
 #define PRISM_TUNE_ROW 0
 #define PRISM_TUNE_COL 1
 #define PRISM_TUNE_SCAN 2  /* contraction tile shape of the FP32 GEMM scan (prism_plan_autotune_scan); a raster
-                              whose rows of 3 or more probes each share one y goes by rows instead, for which
-                              every shape is the same */
+                              whose rows of 3 or more probes each share one y goes by rows, and positions too
+                              far apart to share S values probe by probe, for which every shape is the same */
 #define PRISM_TUNE_SCAN_TC 3  /* ring shape of the tensor-core scan of a 16-bit plan: stages x K values of
                                  its A operand (3 x 96 default, 2 x 128, 4 x 64; split mode 2 x 32 only) */
 #define PRISM_TUNE_MAX_SHAPES 16

@@ -22,13 +22,13 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libprism.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 HEADERS = [os.path.join(CSRC, h) for h in ("fft.cuh", "params.h", "internal.h", "tc.cuh", "scan_common.cuh", "pass_kernels.cuh",
-                                           "tune_shapes.cuh", "tune_pass.cuh", "scan_gemm.cuh", "scan_tc.cuh", "scan_rows.cuh", "launch.cuh",
+                                           "tune_shapes.cuh", "tune_pass.cuh", "scan_gemm.cuh", "scan_tc.cuh", "scan_rows.cuh", "scan_list.cuh", "launch.cuh",
                                            "pass_default.cuh")] + \
     [os.path.join(INCLUDE, "prism.h")]
 CUDA_UNITS = ["kernels_build.cu", "kernels_pass_512.cu", "kernels_pass_1024.cu", "kernels_pass_2048.cu", "kernels_tune.cu",
               "kernels_tune_256.cu", "kernels_tune_512_row.cu", "kernels_tune_512_col.cu", "kernels_tune_1024_row.cu",
               "kernels_tune_1024_col.cu", "kernels_tune_2048_row.cu", "kernels_tune_2048_col.cu", "kernels_scan.cu",
-              "kernels_scan_rows.cu", "kernels_scan_rows_64.cu",
+              "kernels_scan_rows.cu", "kernels_scan_rows_64.cu", "kernels_scan_list.cu",
               "kernels_tune_scan.cu", "kernels_tc.cu", "kernels_tc_tune.cu", "noalloc.cu"]
 HOST_UNITS = ["engine.cpp", "server.cpp"]
 

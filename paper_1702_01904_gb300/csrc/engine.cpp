@@ -951,6 +951,8 @@ extern "C" int prism_build_smatrix_host(prism_plan *P, const float *V_host) {
 static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) {
     const bool split = P->prec == PRISM_PRECISION_FP16X2;
     if ((P->prec != PRISM_PRECISION_FP32 && !split) || sc->px < 3 || sc->py < 1) return;
+    // (up to 24 FP32 probes are as fast probe by probe, or faster: 4 x 4 of 129 beams 66 us by rows, 36 so)
+    if (!split && P->nw < 128 && (long long)sc->px * sc->py <= 24) return;
     double xmin = sc->x0[0], xmax = sc->x0[0], ymin = sc->y0[0], ymax = sc->y0[0];
     for (int r = 0; r < sc->py; ++r) {
         const double *x = sc->x0 + (size_t)r * sc->px, *y = sc->y0 + (size_t)r * sc->px;
@@ -1007,6 +1009,42 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
     a.rows_y0 = split ? gy : 0;
     a.rows_pitch = split ? cols : P->nxs;
     a.rows_ry = split ? rows : P->nys;
+}
+
+// Whether the scan goes probe by probe (scan_list.cuh): FP32, not by raster rows, and
+//  - at least half of the 4 x 8 blocks of the general scan (scan_gemm.cuh) could not share a union tile (its
+//    test, by the extent of their positions: larger in pixels than their windows together), or
+//  - the raster does not fill blocks (fewer than 8 rows of it: a list of positions fills 4 slots of a
+//    block's 32), or has fewer than 2048 probes; of 128-pixel windows fewer than 64.
+// Measured, blocks against probe by probe: 900 scattered probes 1.32 -> 0.34 ms (129 beams, 64-pixel windows),
+// 2.80 -> 0.47 (213), 10 of them 317 -> 35 us; a dense line of 900 0.45 -> 0.33; a rotated 30 x 30 raster
+// 0.38 -> 0.26, but 63 x 63 0.86 -> 1.13; 128-pixel windows: 10 probes 0.42 -> 0.23, 100 on a line
+// 0.92 -> 1.39, 900 scattered 24.9 -> 14.7.
+static void position_list(const prism_plan *P, const prism_scan *sc, ScanArgs &a) {
+    if (P->prec != PRISM_PRECISION_FP32 || a.rows_lp > 0 || !scan_list_supported(P->nw, P->nwy, P->nbeams)) return;
+    const long long n = (long long)sc->px * sc->py;
+    const bool large = P->nw >= 128;
+    if (n > 0 && (large ? n < 64 : sc->py < 8 || n < 2048)) {
+        a.list = 1;
+        return;
+    }
+    long long apart = 0, blocks = 0;
+    for (int by = 0; by < sc->py; by += 8)
+        for (int bx = 0; bx < sc->px; bx += 4) {
+            const int ny = std::min(8, sc->py - by), nx = std::min(4, sc->px - bx);
+            double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
+            for (int j = by; j < by + ny; ++j)
+                for (int i = bx; i < bx + nx; ++i) {
+                    const size_t q = (size_t)j * sc->px + i;
+                    x0 = std::min(x0, sc->x0[q]);
+                    x1 = std::max(x1, sc->x0[q]);
+                    y0 = std::min(y0, sc->y0[q]);
+                    y1 = std::max(y1, sc->y0[q]);
+                }
+            ++blocks;
+            apart += ((x1 - x0) / a.px_s + P->nw) * ((y1 - y0) / a.py_s + P->nwy) > (double)nx * ny * P->nw * P->nwy;
+        }
+    a.list = blocks > 0 && 2 * apart >= blocks;
 }
 
 static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_scan *sc, const prism_detector *det,
@@ -1128,6 +1166,7 @@ static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_sca
     a.n_fold16 = det ? (int)P->fold_n : 0;
     a.tw = P->tw64;
     raster_rows(P, sc, a);
+    position_list(P, sc, a);
     return PRISM_OK;
 }
 
@@ -1174,6 +1213,10 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
         *grid = 1;
         return PRISM_OK;
     }
+    if (a.list) {
+        *grid = 1;
+        return PRISM_OK;
+    }
     if (P->prec == PRISM_PRECISION_FP32) {
         const int sh = gemm_shape(P);
         *grid = scan_gemm_grid(P->nw, P->nwy, sh, P->nbeams, a.scan_px, a.scan_py);
@@ -1201,6 +1244,7 @@ static int scan_go(prism_plan *P, const ScanArgs &a, int grid) {
         if (!rc) P->launches += 2 * ((a.scan_py + a.rows_chunk - 1) / a.rows_chunk) - 1 + a.rows_unpack;
         return rc;
     }
+    if (a.list) return plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_list(P->nw, P->nwy, a, P->stream); });
     if (P->prec == PRISM_PRECISION_FP32)
         return plan_launch(P, PRISM_K_SCAN, [&] {
             return grid > 0 ? launch_scan_gemm(P->nw, P->nwy, gemm_shape(P), grid, a, P->stream)
@@ -1933,9 +1977,9 @@ extern "C" int prism_plan_autotune_scan(prism_plan *P, const prism_probe *probe,
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
-    // a scan by raster rows has no contraction blocks: timed once, the same for every shape, and the
-    // plan's shape stays (position lists use it)
-    const bool rows = a.rows_lp > 0;
+    // a scan by raster rows or probe by probe has no contraction blocks: timed once, the same for every
+    // shape, and the plan's shape stays
+    const bool rows = a.rows_lp > 0 || a.list;
     const int kept = P->scan_shape;
     int best = rows ? kept : 0;
     double best_ms = -1.0;

@@ -135,6 +135,7 @@ struct ScanArgs {
     int rows_unpack;
     int rows_lp;               // probes per CTA
     int rows_0, rows_n;        // set per launch: first raster row, raster rows
+    int list;                  // 1: probe by probe (scan_list.cuh), positions too far apart to share S values
     const uint16_t *fold16;    // the bins over the quadrant 0 <= kx <= nw_x/2, 0 <= ky <= nw_y/2: CSR offsets
                                // [nbins + 1], then the lists (ky * (nw_x/2 + 1) + kx); 16-byte aligned
     int n_fold16;              // its entries, padded to 8 (0: no bins)
@@ -224,6 +225,9 @@ size_t scan_gemm_cnt_bytes(int grid);
 // or sizes are not for it), launch
 size_t scan_rows_unpack_bytes(const ScanArgs &a);  // bytes of rows_src where it is unpacked
 int scan_rows_lp(int nwx, int nwy, int m, int max_beams, int lists, int px, int rows);
+// the position-list scan (scan_list.cuh): whether it takes these windows and beams, launch
+bool scan_list_supported(int nwx, int nwy, int n_beams);
+cudaError_t launch_scan_list(int nwx, int nwy, const ScanArgs &a, cudaStream_t s);
 cudaError_t launch_scan_rows(int nwx, int nwy, const ScanArgs &a, cudaStream_t s);
 cudaError_t launch_shift(const ShiftArgs &a, cudaStream_t s);
 cudaError_t launch_bins(const BinArgs &a, cudaStream_t s);

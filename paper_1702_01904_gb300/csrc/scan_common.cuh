@@ -182,9 +182,10 @@ struct ExSize {
     static constexpr int value = EXR > EXC ? EXR : EXC;
 };
 
+// the 2-D FFTs of the windows alone
 template <int NWX, int NWY, int BLOCK, int G, int PW>
-__device__ void window_epilogue(const ScanArgs &a, float2 *win, float2 *ex, const float2 *twx, const float2 *twy,
-                                int nwin, const int *oidx, int tid, const uint16_t *sidx = nullptr) {
+__device__ __forceinline__ void window_transforms(const ScanArgs &a, float2 *win, float2 *ex, const float2 *twx, const float2 *twy,
+                                                  int nwin, int tid) {
     {
         using FS = FftShape<NWX>;
         using Fwd = FwdFft<NWX>;
@@ -234,6 +235,12 @@ __device__ void window_epilogue(const ScanArgs &a, float2 *win, float2 *ex, cons
         }
     }
     __syncthreads();
+}
+
+// the outputs of transformed windows
+template <int NWX, int NWY, int BLOCK, int G, int PW>
+__device__ __forceinline__ void window_outputs(const ScanArgs &a, const float2 *win, int nwin, const int *oidx, int tid,
+                                               const uint16_t *sidx = nullptr) {
     // u = ky * NWX + kx: the row is u >> LNW, LNW = log2(NWX)
     constexpr int LNW = NWX == 8 ? 3 : NWX == 16 ? 4 : NWX == 32 ? 5 : NWX == 64 ? 6 : NWX == 128 ? 7 : -1;
     static_assert(LNW > 0 && (1 << LNW) == NWX, "window widths 8 ... 128");
@@ -284,6 +291,13 @@ __device__ void window_epilogue(const ScanArgs &a, float2 *win, float2 *ex, cons
             *o = a.accumulate ? *o + a.acc_w * val : val;
         }
     }
+}
+
+template <int NWX, int NWY, int BLOCK, int G, int PW>
+__device__ void window_epilogue(const ScanArgs &a, float2 *win, float2 *ex, const float2 *twx, const float2 *twy,
+                                int nwin, const int *oidx, int tid, const uint16_t *sidx = nullptr) {
+    window_transforms<NWX, NWY, BLOCK, G, PW>(a, win, ex, twx, twy, nwin, tid);
+    window_outputs<NWX, NWY, BLOCK, G, PW>(a, win, nwin, oidx, tid, sidx);
 }
 
 }  // namespace prism

@@ -1,0 +1,188 @@
+// scan_list.cuh -- the FP32 PRISM scan of positions too far apart to share S values (k_scan_list): scattered
+// position lists, sparse rasters.  One CTA per probe: a thread owns a few window pixels and walks the beams,
+// several beams' loads in flight; the window then goes through shared memory for its transform and bins.
+//
+// Bound by the S values read, B nw^2 8 bytes per probe once from the L2 (900 scattered probes of 129 beams
+// and 64-pixel windows: 3.8 GB in 0.34 ms).  The blocks of scan_gemm.cuh run such probes one after another
+// with one warp in eight at work, and a list of positions fills 4 of their 32 slots: 1.32 ms for those 900,
+// 0.32 for 10 of them (35 us here).  900 jittered positions of 32 x 16 windows and 25 beams: 69 -> 20 us on
+// the device.
+// Few probes: a cluster of up to 8 CTAs shares a probe's beams, and their windows are added in the first
+// one's shared memory, rank by rank.  Bins of short lists (up to 1024-pixel windows) take a thread each
+// (4000 probes of 16 x 16 windows: 162 us with a warp each, 89 so).
+#pragma once
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+
+#include "fft.cuh"
+#include "params.h"
+#include "scan_common.cuh"
+
+namespace prism {
+
+template <int NWX, int NWY>
+struct ListCfg {
+    static constexpr int NP = NWX * NWY;
+    static constexpr int BLOCK = NP <= 1024 ? 128 : NP <= 4096 ? 256 : 512;
+    static constexpr int PIX = NP / BLOCK;                    // window pixels per thread
+    // a batch of loads: U beams' values of a thread's pixels, or, of 32 pixels, a quarter of one beam's (the
+    // batch after the one being summed is in flight)
+    static constexpr int U = PIX >= 16 ? 1 : 16 / PIX;
+    static constexpr int PB = PIX > 16 ? 8 : PIX;             // pixels of a batch
+    static constexpr int NB = PIX / PB;                       // batches per U beams
+    static constexpr int PW = NWX + 4;                        // window row pitch (bank spread)
+    static constexpr int EX = ExSize<NWX, NWY, BLOCK>::value;
+    static constexpr size_t FIXED = (size_t)(NWY * PW + EX + NWX + NWY) * sizeof(float2);
+    static_assert(BLOCK % NWX == 0 || NWX % BLOCK == 0, "a thread's pixels lie in one column");
+};
+
+template <int NWX, int NWY>
+__global__ void __launch_bounds__(ListCfg<NWX, NWY>::BLOCK) k_scan_list(const __grid_constant__ ScanArgs a) {
+    using C = ListCfg<NWX, NWY>;
+    constexpr int BLOCK = C::BLOCK, PIX = C::PIX, U = C::U, PW = C::PW, RS = BLOCK / NWX;  // rows between a thread's pixels
+    extern __shared__ __align__(16) float2 sm_list[];
+    float2 *win = sm_list;              // [NWY][PW]
+    float2 *ex = win + NWY * PW;
+    float2 *twx = ex + C::EX, *twy = twx + NWX;
+    float2 *alpha = twy + NWY;          // [n_beams]
+    const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int cr = (int)cl.block_rank(), cn = (int)cl.num_blocks();
+    const int tid = threadIdx.x, p = blockIdx.x / cn;
+    const int bb = cr * a.n_beams / cn, be = (cr + 1) * a.n_beams / cn;  // this CTA's beams
+    for (int i = tid; i < NWX; i += BLOCK) twx[i] = a.tw_fwd[i];
+    for (int i = tid; i < NWY; i += BLOCK) twy[i] = a.tw_fwd_y[i];
+    const double x0 = a.x0[p], y0 = a.y0[p];
+    for (int b = bb + tid; b < be; b += BLOCK) {
+        double c = a.qx[b] * (x0 - a.shift_x) + a.qy[b] * (y0 - a.shift_y);
+        c -= rint(c);
+        float s, co;
+        sincospif(-2.0f * (float)c, &s, &co);
+        alpha[b] = cmul(__ldg(a.base + b), make_float2(co, s));
+    }
+    const int sx = ((int)floor(x0 / a.px_s + 0.5) - NWX / 2) & (a.nx_s - 1);
+    const int sy = ((int)floor(y0 / a.py_s + 0.5) - NWY / 2) & (a.ny_s - 1);
+    const int wx = tid % NWX, wy = tid / NWX;  // this thread's pixels: column wx, rows wy + RS k
+    const float2 *Sx = a.S + ((sx + wx) & (a.nx_s - 1));
+    const size_t bstride = (size_t)a.ny_s * a.nx_s;
+    float2 acc[PIX];
+#pragma unroll
+    for (int k = 0; k < PIX; ++k) acc[k] = make_float2(0.f, 0.f);
+    __syncthreads();
+    constexpr int PB = C::PB, NB = C::NB;
+    auto load = [&](float2 (&s)[U][PB], int b0, int h) {  // batch h of beams b0 ... b0 + U - 1
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+            if (b0 + i < be) {
+                const float2 *Sb = Sx + (size_t)(b0 + i) * bstride;
+#pragma unroll
+                for (int k = 0; k < PB; ++k) s[i][k] = __ldg(Sb + (size_t)((sy + wy + RS * (h * PB + k)) & (a.ny_s - 1)) * a.nx_s);
+            }
+    };
+    float2 cur[U][PB], nxt[U][PB];
+    load(cur, bb, 0);
+#pragma unroll 1
+    for (int b0 = bb; b0 < be; b0 += U) {
+#pragma unroll
+        for (int h = 0; h < NB; ++h) {
+            if (h + 1 < NB) load(nxt, b0, h + 1);
+            else load(nxt, b0 + U, 0);
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                if (b0 + i < be) {
+                    const float2 al = alpha[b0 + i];
+#pragma unroll
+                    for (int k = 0; k < PB; ++k) {
+                        float2 &c = acc[h * PB + k];
+                        const float2 s = cur[i][k];
+                        c.x = fmaf(al.x, s.x, fmaf(-al.y, s.y, c.x));
+                        c.y = fmaf(al.x, s.y, fmaf(al.y, s.x, c.y));
+                    }
+                }
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+#pragma unroll
+                for (int k = 0; k < PB; ++k) cur[i][k] = nxt[i][k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < PIX; ++k) win[(wy + RS * k) * PW + wx] = acc[k];
+    if (cn > 1) {
+        // every rank's window is written; the first adds the others' to its own, then they may leave
+        cl.sync();
+        if (cr == 0) {
+            for (int r = 1; r < cn; ++r) {
+                const float2 *o = cl.map_shared_rank(win, r);
+#pragma unroll
+                for (int k = 0; k < PIX; ++k) acc[k] = cadd(acc[k], o[(wy + RS * k) * PW + wx]);
+            }
+#pragma unroll
+            for (int k = 0; k < PIX; ++k) win[(wy + RS * k) * PW + wx] = acc[k];
+        }
+        cl.sync();
+        if (cr != 0) return;
+    }
+    __syncthreads();
+    window_transforms<NWX, NWY, BLOCK, 1, PW>(a, win, ex, twx, twy, 1, tid);
+    __shared__ int row;
+    if constexpr (C::NP <= 1024) {
+        // short lists: a thread per bin
+        if (tid == 0) row = p;
+        __syncthreads();
+        window_outputs<NWX, NWY, BLOCK, 1, PW>(a, win, 1, &row, tid);
+        return;
+    }
+    constexpr int LNW = NWX == 16 ? 4 : NWX == 32 ? 5 : NWX == 64 ? 6 : 7;
+    if (a.cbed) {
+        const float fnorm = (float)a.inv_norm;
+        for (int u = tid; u < C::NP; u += BLOCK) {
+            const float2 z = win[(u >> LNW) * PW + (u & (NWX - 1))];
+            a.cbed[(size_t)p * C::NP + u] = (z.x * z.x + z.y * z.y) * fnorm;
+        }
+    }
+    if (!a.out) return;
+    // a warp per annular bin: lanes over its pixel list, FP32 partial sums, a fixed xor tree, FP64 scale
+    const int lane = tid & 31;
+    for (int k = tid >> 5; k < a.nbins; k += BLOCK / 32) {
+        float s = 0.f;
+        const int e = __ldg(a.bin_off + k + 1);
+        for (int i = __ldg(a.bin_off + k) + lane; i < e; i += 32) {
+            const int u = __ldg(a.bin_idx + i);
+            const float2 z = win[(u >> LNW) * PW + (u & (NWX - 1))];
+            s = fmaf(z.x, z.x, fmaf(z.y, z.y, s));
+        }
+        s = warp_sum(s);
+        if (lane == 0) {
+            const float val = (float)((double)s * a.inv_norm);
+            float *o = a.out + (size_t)p * a.nbins + k;
+            *o = a.accumulate ? *o + a.acc_w * val : val;
+        }
+    }
+}
+
+template <int NWX, int NWY>
+static size_t list_smem(int n_beams) {
+    return ListCfg<NWX, NWY>::FIXED + (size_t)n_beams * sizeof(float2);
+}
+
+template <int NWX, int NWY>
+static cudaError_t list_launch(const ScanArgs &a, cudaStream_t s) {
+    cudaError_t e = allow_max_dynamic_smem(k_scan_list<NWX, NWY>);
+    if (e != cudaSuccess) return e;
+    // CTAs per probe: as many (up to 8, of 4 beams or more) as leave two CTAs per SM or fewer
+    int cn = 1;
+    while (cn < 8 && (long long)a.n_probes * cn * 2 <= 2 * 152 && a.n_beams >= 8 * cn) cn *= 2;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cn;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)(a.n_probes * cn));
+    c.blockDim = dim3(ListCfg<NWX, NWY>::BLOCK);
+    c.dynamicSmemBytes = list_smem<NWX, NWY>(a.n_beams);
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k_scan_list<NWX, NWY>, a);
+}
+
+}  // namespace prism

@@ -55,7 +55,7 @@ def raster(kind, cell, px, py, step):
     (256, 16.0, 1, 0, 14.0),    # 128 x 128
     (256, 16.0, 4, 0, 1.0),     # one beam
 ])
-@pytest.mark.parametrize("kind,px,py,step", [("plain", 3, 5, 0.3), ("wrap", 33, 3, 0.21), ("serpentine", 9, 6, 0.05),
+@pytest.mark.parametrize("kind,px,py,step", [("plain", 3, 9, 0.3), ("wrap", 33, 3, 0.21), ("serpentine", 9, 6, 0.05),
                                              ("skew", 17, 9, 0.4), ("wrap", 7, 4, 2.7), ("plain", 64, 2, 0.11)])
 def test_rows_equal_the_general_scan(n, cell, f, f_y, alpha, kind, px, py, step):
     sim = plan(n, cell, f, f_y, alpha, 5)
@@ -120,4 +120,40 @@ def test_rows_of_value_and_remainder_storage(n, cell, f, alpha, kind, px, py, st
     close(got, ref, sim.info.n_beams, 2.0 ** -20)
     cb = sim.scan_cbed(probe, x0, y0, px=px, py=py).cpu().numpy()
     close(cb, sim.scan_cbed(probe, x0, y0).cpu().numpy(), sim.info.n_beams, 2.0 ** -20)
+    sim.close()
+
+
+@pytest.mark.parametrize("n,cell,f,f_y,alpha", [(64, 8.0, 2, 0, 20.0), (64, 8.0, 2, 1, 20.0), (128, 12.8, 1, 4, 20.0), (256, 16.0, 4, 0, 20.0),
+                                                (256, 16.0, 4, 2, 9.0), (256, 12.5, 2, 0, 28.0), (256, 16.0, 1, 0, 14.0), (256, 16.0, 4, 0, 1.0)])
+@pytest.mark.parametrize("count", [1, 2, 19, 60, 170])
+def test_position_lists(n, cell, f, f_y, alpha, count):
+    # probe by probe (one CTA or a cluster of up to 8 per probe) against FP64 sums of the same S-matrix, beams
+    # from one to several hundred; positions wrap and are negative
+    sim = plan(n, cell, f, f_y, alpha, 9)
+    i = sim.info
+    r = np.random.default_rng(4)
+    x0, y0 = r.uniform(-cell, 2 * cell, count), r.uniform(-cell, 2 * cell, count)
+    got = sim.scan_cbed(P.make_probe(20.0, 25.0), x0, y0).cpu().numpy()
+    m, k = sim.beams()
+    fy = f_y or f
+    lam = P.prism_wavelength(300.0)
+    qx, qy = m * f / cell, k * fy / cell
+    inside = (lam * qx) ** 2 + (lam * qy) ** 2 <= 0.02 ** 2 * (1 + 1e-12)
+    A = inside * np.exp(-1j * np.pi * lam * (qx ** 2 + qy ** 2) * 25.0)
+    S = sim.smatrix().cpu().numpy().astype(np.complex128)
+    for p in sorted({0, count // 2, count - 1}):
+        a = A * np.exp(-2j * np.pi * (qx * x0[p] + qy * y0[p]))
+        ix = (int(np.floor(x0[p] / (cell / i.nx_s) + 0.5)) - i.nw_x // 2 + np.arange(i.nw_x)) % i.nx_s
+        iy = (int(np.floor(y0[p] / (cell / i.ny_s) + 0.5)) - i.nw_y // 2 + np.arange(i.nw_y)) % i.ny_s
+        psi = np.tensordot(a, S[:, iy[:, None], ix[None, :]], axes=(0, 0))
+        ref = np.abs(np.fft.fft2(psi)) ** 2 / ((i.nw_x * i.nw_y) ** 2 * inside.sum())
+        # (the FP32 coefficients besides: phase and product, 2^-22 of each)
+        close(got[p], ref, i.n_beams, 2.0 ** -22)
+    det = P.make_detector(0.0, 2.0, 40)
+    out = sim.scan(P.make_probe(20.0, 25.0), x0, y0, det).cpu().numpy()
+    wx = np.fft.fftfreq(i.nw_x, 1.0 / i.nw_x) * f / cell
+    wy = np.fft.fftfreq(i.nw_y, 1.0 / i.nw_y) * fy / cell
+    b = np.floor(1000.0 * lam * np.sqrt(wx[None, :] ** 2 + wy[:, None] ** 2) / 2.0).astype(int)
+    ref = np.stack([got[:, b == j].astype(np.float64).sum(1) for j in range(40)], axis=1)
+    close(out, ref, i.n_beams)
     sim.close()
