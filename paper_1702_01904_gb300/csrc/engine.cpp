@@ -413,6 +413,7 @@ struct prism_plan {
     int rows_m = 0, rows_maxn = 0;
     float2 *rows_w = nullptr;  // sums over n of the raster-row scan
     size_t rows_cap = 0;
+    bool rows_attrs = false, list_attrs = false;  // the kernels' shared-memory limits have been set
     float2 *rows_s = nullptr;  // what the windows reach of a value + remainder S-matrix, unpacked
     size_t rows_s_cap = 0;
     // grown on demand
@@ -1075,14 +1076,22 @@ static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_sca
     }
     const long long Pn = (long long)sc->px * sc->py;
     if ((rc = grow(P->arena, (void **)&P->pos, &P->pos_cap, std::max<size_t>(16, (size_t)Pn * 2 * sizeof(double))))) return rc;
-    if (Pn > 0) {
-        // pageable copy of the caller's arrays: cudaMemcpyAsync stages pageable memory before it returns
+    {
+        // positions and coefficients: as kernel parameters where they are small, else as pageable copies
+        // (cudaMemcpyAsync stages pageable memory before it returns)
         std::vector<double> xy((size_t)Pn * 2);
-        std::memcpy(xy.data(), sc->x0, Pn * sizeof(double));
-        std::memcpy(xy.data() + Pn, sc->y0, Pn * sizeof(double));
-        CUDA_TRY(cudaMemcpyAsync(P->pos, xy.data(), xy.size() * sizeof(double), cudaMemcpyHostToDevice, P->stream));
+        if (Pn > 0) {
+            std::memcpy(xy.data(), sc->x0, Pn * sizeof(double));
+            std::memcpy(xy.data() + Pn, sc->y0, Pn * sizeof(double));
+        }
+        if (2 * Pn + B <= PUT_LARGE) {
+            const cudaError_t e = launch_put(P->pos, xy.data(), (int)(2 * Pn), P->base, base.data(), B, P->stream);
+            if (e != cudaSuccess) return fail(PRISM_ERR_CUDA, std::string("position upload: ") + cudaGetErrorString(e));
+        } else {
+            if (Pn > 0) CUDA_TRY(cudaMemcpyAsync(P->pos, xy.data(), xy.size() * sizeof(double), cudaMemcpyHostToDevice, P->stream));
+            CUDA_TRY(cudaMemcpyAsync(P->base, base.data(), B * sizeof(float2), cudaMemcpyHostToDevice, P->stream));
+        }
     }
-    CUDA_TRY(cudaMemcpyAsync(P->base, base.data(), B * sizeof(float2), cudaMemcpyHostToDevice, P->stream));
     // window bin map (q = k f / cell on the window grid), cached per detector
     if (det && (P->det_nbins != det->nbins || P->det_key[0] != det->start_mrad || P->det_key[1] != det->step_mrad)) {
         std::vector<int> off, idx;
@@ -1167,6 +1176,8 @@ static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_sca
     a.tw = P->tw64;
     raster_rows(P, sc, a);
     position_list(P, sc, a);
+    // (which kernels, and so their limits, depends on the plan's windows and beams alone)
+    a.attrs_set = a.rows_lp > 0 ? P->rows_attrs : P->list_attrs;
     return PRISM_OK;
 }
 
@@ -1240,11 +1251,16 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
 static int scan_go(prism_plan *P, const ScanArgs &a, int grid) {
     if (a.rows_lp > 0) {
         const int rc = plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_rows(P->nw, P->nwy, a, P->stream); });
+        P->rows_attrs = P->rows_attrs || !rc;
         // two kernels per chunk of rows, and the unpacking
         if (!rc) P->launches += 2 * ((a.scan_py + a.rows_chunk - 1) / a.rows_chunk) - 1 + a.rows_unpack;
         return rc;
     }
-    if (a.list) return plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_list(P->nw, P->nwy, a, P->stream); });
+    if (a.list) {
+        const int rc = plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_list(P->nw, P->nwy, a, P->stream); });
+        P->list_attrs = P->list_attrs || !rc;
+        return rc;
+    }
     if (P->prec == PRISM_PRECISION_FP32)
         return plan_launch(P, PRISM_K_SCAN, [&] {
             return grid > 0 ? launch_scan_gemm(P->nw, P->nwy, gemm_shape(P), grid, a, P->stream)

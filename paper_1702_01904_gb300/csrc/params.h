@@ -135,6 +135,7 @@ struct ScanArgs {
     int rows_unpack;
     int rows_lp;               // probes per CTA
     int rows_0, rows_n;        // set per launch: first raster row, raster rows
+    int attrs_set;             // the row or list kernels' shared-memory limits are set (by this plan, before)
     int list;                  // 1: probe by probe (scan_list.cuh), positions too far apart to share S values
     const uint16_t *fold16;    // the bins over the quadrant 0 <= kx <= nw_x/2, 0 <= ky <= nw_y/2: CSR offsets
                                // [nbins + 1], then the lists (ky * (nw_x/2 + 1) + kx); 16-byte aligned
@@ -189,6 +190,16 @@ struct BinArgs {
     const int *err;            // optional device error word of the passes: non-zero -> the bins are NaN
 };
 
+// Small tables that travel as kernel parameters (launch_put): `data` holds n0 8-byte words for dst0, then
+// n1 for dst1
+constexpr int PUT_SMALL = 448, PUT_LARGE = 2000;  // words: about 4 and 16 KB of parameters
+template <int N>
+struct PutArgs {
+    unsigned long long *dst0, *dst1;
+    int n0, n1;
+    unsigned long long data[N];
+};
+
 // launchers (kernels_build.cu, kernels_scan.cu); return cudaSuccess or the launch error
 cudaError_t launch_transmission(const float *V, float2 *t, size_t n, double sigma_cycles, cudaStream_t s);
 // first-slice rows of beams beam0 .. beam0+nb-1 from T0 = FFT_x(t_0) [ny][nx] (kept columns only)
@@ -231,6 +242,9 @@ cudaError_t launch_scan_list(int nwx, int nwy, const ScanArgs &a, cudaStream_t s
 cudaError_t launch_scan_rows(int nwx, int nwy, const ScanArgs &a, cudaStream_t s);
 cudaError_t launch_shift(const ShiftArgs &a, cudaStream_t s);
 cudaError_t launch_bins(const BinArgs &a, cudaStream_t s);
+// two host arrays of 8-byte words to the device in one launch (n0 + n1 <= PUT_LARGE); the arrays are read
+// before it returns
+cudaError_t launch_put(void *dst0, const void *src0, int n0, void *dst1, const void *src1, int n1, cudaStream_t s);
 cudaError_t launch_bin_lists(const BinListArgs &a, cudaStream_t s);
 cudaError_t launch_probe_base(const ProbeBaseArgs &a, size_t npix, cudaStream_t s);
 cudaError_t launch_tc_selftest(float *out, int *status, cudaStream_t s);

@@ -166,8 +166,10 @@ static size_t list_smem(int n_beams) {
 
 template <int NWX, int NWY>
 static cudaError_t list_launch(const ScanArgs &a, cudaStream_t s) {
-    cudaError_t e = allow_max_dynamic_smem(k_scan_list<NWX, NWY>);
-    if (e != cudaSuccess) return e;
+    if (!a.attrs_set) {
+        const cudaError_t e = allow_max_dynamic_smem(k_scan_list<NWX, NWY>);
+        if (e != cudaSuccess) return e;
+    }
     // CTAs per probe: as many (up to 8, of 4 beams or more) as leave two CTAs per SM or fewer
     int cn = 1;
     while (cn < 8 && (long long)a.n_probes * cn * 2 <= 2 * 152 && a.n_beams >= 8 * cn) cn *= 2;

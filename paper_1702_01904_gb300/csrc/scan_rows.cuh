@@ -42,14 +42,17 @@ namespace prism {
 constexpr int ROWS_R = 4;    // raster rows per k_rows_sum unit: each S value loaded feeds four sums
 
 // ------------------------------------------------------------------ sums over n, column transforms
-template <int NWY>
+// SMALL: for scans of few units, where a unit's latency counts and not the units an SM holds: more threads
+// (fewer sweeps over the rows) and more loads together
+template <int NWY, bool SMALL = false>
 struct RowsSumCfg {
     using FS = FftShape<NWY>;
-    static constexpr int BLOCK = 192;
+    static constexpr int BLOCK = SMALL ? 256 : 192;
+    static constexpr int MINB = SMALL ? 1 : 3;
     static constexpr int XC = NWY >= 128 ? 8 : 16;       // columns per unit: 64- or 128-byte runs of S and of W
     static constexpr int PAIRS = XC / 2;                 // a thread takes two neighbouring columns
     static constexpr int YSTEP = BLOCK / PAIRS;          // union rows per sweep of the block
-    static constexpr int U = 7;                          // beams whose loads a thread issues together
+    static constexpr int U = SMALL ? 14 : 7;             // beams whose loads a thread issues together
     // A column of one plane and raster row: NWY values, in place the transform's exchange.  The second
     // column of a pair starts 16 banks on (mod 32), so the columns two slots of a half-warp transform
     // fall on different banks; pairs are 4 banks apart (8 for the 4 pairs of 8 columns), so that the
@@ -67,9 +70,9 @@ struct RowsSumCfg {
     }
 };
 
-template <int NWY>
-__global__ void __launch_bounds__(RowsSumCfg<NWY>::BLOCK, 3) k_rows_sum(const __grid_constant__ ScanArgs a) {
-    using C = RowsSumCfg<NWY>;
+template <int NWY, bool SMALL = false>
+__global__ void __launch_bounds__(RowsSumCfg<NWY, SMALL>::BLOCK, RowsSumCfg<NWY, SMALL>::MINB) k_rows_sum(const __grid_constant__ ScanArgs a) {
+    using C = RowsSumCfg<NWY, SMALL>;
     using FS = FftShape<NWY>;
     using Fwd = FwdFft<NWY>;
     constexpr int BLOCK = C::BLOCK, R = ROWS_R, XC = C::XC, T = FS::T, E = FS::E;
@@ -460,19 +463,33 @@ static cudaError_t rows_launch(const ScanArgs &args, cudaStream_t s) {
     if (reinterpret_cast<uintptr_t>(a.rows_src) & 15) return cudaErrorMisalignedAddress;  // pixel pairs are read as one load
     const int kp = rows_kp(a.rows_m);
     const size_t sa = A::smem(a.rows_maxn), sb = B::smem(a.rows_lp, rows_mp(a.rows_m), a.n_fold16);
-    void (*sum)(const ScanArgs) = k_rows_sum<NWY>;
+    // (few units: a chunk of rows makes no more than 2 per SM)
+    const bool small = (long long)(a.rows_cols / A::XC) * (a.rows_m + 1) * ((std::min(a.rows_chunk, a.scan_py) + ROWS_R - 1) / ROWS_R) <= 2 * 152;
+    void (*sum)(const ScanArgs) = small ? k_rows_sum<NWY, true> : k_rows_sum<NWY>;
+    const int sum_block = small ? RowsSumCfg<NWY, true>::BLOCK : A::BLOCK;
+    static_assert(RowsSumCfg<NWY, true>::XC == A::XC && RowsSumCfg<NWY, true>::BUF == A::BUF, "the same unit");
     void (*win)(const ScanArgs) = kp == 4   ? k_rows_window<NWX, NWY, 4>
                                   : kp == 6 ? k_rows_window<NWX, NWY, 6>
                                   : kp == 7 ? k_rows_window<NWX, NWY, 7>
                                             : k_rows_window<NWX, NWY, 8>;
-    cudaError_t e;
-    if ((e = allow_max_dynamic_smem(sum)) != cudaSuccess || (e = allow_max_dynamic_smem(win)) != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (!a.attrs_set && ((e = allow_max_dynamic_smem(k_rows_sum<NWY>)) != cudaSuccess ||
+                         (e = allow_max_dynamic_smem(k_rows_sum<NWY, true>)) != cudaSuccess || (e = allow_max_dynamic_smem(win)) != cudaSuccess))
+        return e;
     const int ngc = (a.scan_px + a.rows_lp - 1) / a.rows_lp;
     for (int r0 = 0; r0 < a.scan_py; r0 += a.rows_chunk) {
         a.rows_0 = r0;
         a.rows_n = std::min(a.rows_chunk, a.scan_py - r0);
         const dim3 ga(a.rows_cols / A::XC, a.rows_m + 1, (a.rows_n + ROWS_R - 1) / ROWS_R);
-        if ((e = launch_chained(sum, ga, A::BLOCK, sa, s, a)) != cudaSuccess) return e;
+        // the first launch is a plain one: the positions and coefficients that both kernels read before
+        // they wait (in their prologues) come from the launch or copies before it
+        if (r0 == 0) {
+            sum<<<ga, sum_block, sa, s>>>(a);
+            e = cudaGetLastError();
+        } else {
+            e = launch_chained(sum, ga, sum_block, sa, s, a);
+        }
+        if (e != cudaSuccess) return e;
         if ((e = launch_chained(win, a.rows_n * ngc, B::BLOCK, sb, s, a)) != cudaSuccess) return e;
     }
     return cudaSuccess;

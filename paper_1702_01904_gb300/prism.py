@@ -239,10 +239,18 @@ def make_probe(alpha_mrad, c1=0.0, c3=0.0, tilt_x=0.0, tilt_y=0.0):
     return PrismProbe(alpha_mrad, c1, c3, tilt_x, tilt_y)
 
 
+def _doubles(a):
+    """A C-contiguous float64 array as the value of a POINTER(c_double) field."""
+    try:
+        return (c_double * a.size).from_buffer(a)
+    except (TypeError, ValueError):  # read-only or empty
+        return a.ctypes.data_as(POINTER(c_double))
+
+
 def make_scan(px, py, x0, y0):
     x0 = np.ascontiguousarray(x0, dtype=np.float64)
     y0 = np.ascontiguousarray(y0, dtype=np.float64)
-    s = PrismScan(px, py, x0.ctypes.data_as(POINTER(c_double)), y0.ctypes.data_as(POINTER(c_double)))
+    s = PrismScan(px, py, _doubles(x0), _doubles(y0))
     s._keep = (x0, y0)
     return s
 
