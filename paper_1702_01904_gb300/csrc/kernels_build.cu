@@ -95,7 +95,7 @@ cudaError_t launch_plane(const float2 *T0, float2 *wave, const int *beam_mn, int
     if (nb <= 0) return cudaSuccess;
     if ((nx & (nx - 1)) || (ny & (ny - 1))) return cudaErrorInvalidValue;  // the masks need powers of two
     const int rows = nb * ny;
-    return launch_chained(k_plane, rows < 152 * 8 ? rows : 152 * 8, 256, 0, s, T0, wave, beam_mn, beam0, nb, nx, ny, f, f_y, kx_half);
+    return launch_chained_if((long long)rows * nx <= CHAIN_POINTS, k_plane, rows < 152 * 8 ? rows : 152 * 8, 256, 0, s, T0, wave, beam_mn, beam0, nb, nx, ny, f, f_y, kx_half);
 }
 
 cudaError_t launch_transmission(const float *V, float2 *t, size_t n, double sigma_cycles, cudaStream_t s) {

@@ -9,7 +9,9 @@
 // its predecessor have finished: what a prologue reads must have been complete before the chain began, at a
 // plain launch or a copy.)
 // Measured: S-matrix build of a 256^2 cell 195 -> 152 us, multislice of 256 probes there 676 -> 624 us, a
-// 512^2 simulation 3.92 -> 3.84 ms; no difference on launches of 100 us and more (1024^2).
+// 512^2 simulation (120 us passes of 56 M points) 3.92 -> 3.84 ms; no difference at 1024^2 with 129 beams
+// (200 to 300 us passes of 135 M points), and 15.28 -> 15.50 ms for an 8-slice build of 529 beams there (0.8
+// and 1.2 ms passes).  So the passes chain up to CHAIN_POINTS points.
 // Under stream capture the launches are plain ones.
 #pragma once
 #include <cuda_runtime.h>
@@ -19,10 +21,12 @@ namespace prism {
 __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
+constexpr long long CHAIN_POINTS = 1LL << 26;
+
 template <class... P, class... A>
-static cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args) {
+static cudaError_t launch_chained_if(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();  // (as if captured: a plain launch)
+    if (chain && cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();  // (as if captured: a plain launch)
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
@@ -34,6 +38,10 @@ static cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
     c.attrs = &at;
     c.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, args...);
+}
+template <class... P, class... A>
+static cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args) {
+    return launch_chained_if(true, kernel, grid, block, smem, s, args...);
 }
 
 }  // namespace prism

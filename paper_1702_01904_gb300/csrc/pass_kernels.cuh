@@ -329,7 +329,7 @@ static cudaError_t row_go_bl(const RowArgs &a, cudaStream_t s) {
     cudaError_t e = persistent_grid(k_row<NX, MODE, THR, STG, BL, TM, RV>, C::THREADS, C::SMEM, (a.n_rows + C::SLOTS - 1) / C::SLOTS,
                                     &grid, C::PERSIST);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_row<NX, MODE, THR, STG, BL, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
+    return launch_chained_if((long long)a.n_rows * NX <= CHAIN_POINTS, k_row<NX, MODE, THR, STG, BL, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
 }
 
 // TM: bulk staging where it applies (the compile-time band, one slot per warp, rows read from the
@@ -677,12 +677,12 @@ static cudaError_t col_go(const ColArgs &a, cudaStream_t s) {
             if (a.band4) {
                 e = persistent_grid(k_col<NY, MODE, WC, STG, MB, true, TM, RV>, C::THREADS, C::SMEM, work, &grid, C::PERSIST);
                 if (e != cudaSuccess) return e;
-                return launch_chained(k_col<NY, MODE, WC, STG, MB, true, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
+                return launch_chained_if((long long)a.batch * a.nx * NY <= CHAIN_POINTS, k_col<NY, MODE, WC, STG, MB, true, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
             }
         }
         e = persistent_grid(k_col<NY, MODE, WC, STG, MB, false, TM, RV>, C::THREADS, C::SMEM, work, &grid, C::PERSIST);
         if (e != cudaSuccess) return e;
-        return launch_chained(k_col<NY, MODE, WC, STG, MB, false, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
+        return launch_chained_if((long long)a.batch * a.nx * NY <= CHAIN_POINTS, k_col<NY, MODE, WC, STG, MB, false, TM, RV>, grid, C::THREADS, C::SMEM, s, a);
     }
 }
 
