@@ -1465,7 +1465,7 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
         }
     }
     CUtensorMap map8, map4, out8, out4;
-    const bool maps_ok = (ny == 256 || ny == 512 || ny == 1024) && encode_wave_maps(map8, map4, out8, out4, wave, nx, ny, Pb);
+    const bool maps_ok = ny >= 256 && encode_wave_maps(map8, map4, out8, out4, wave, nx, ny, Pb);
     {
         // the probe phase uses r0 - h tan(theta) (zero without tilt)
         std::vector<double> xy((size_t)Pn * 2);
@@ -1527,16 +1527,16 @@ extern "C" int multislice_scan_run(const prism_grid *grid, const float *V_dev, c
             ca.kx_half = p + 1 == g.n_slices ? 0 : kx_half;
             ca.band4 = T.band4;
             const int cs = p + 1 < g.n_slices ? tune_col_default(ny, (long long)(kx_half > 0 ? 2 * kx_half : nx) * nb, maps_ok, false) : -1;
+            if (maps_ok && p + 1 < g.n_slices) {
+                ca.wave_map = map8;
+                ca.wave_map4 = map4;
+                ca.out_map = out8;
+                ca.out_map4 = out4;
+                ca.wave_map_ok = 1;
+                ca.tile_ctr = err + 1;
+                ca.err = err;
+            }
             if (cs >= 0) {
-                if (maps_ok) {
-                    ca.wave_map = map8;
-                    ca.wave_map4 = map4;
-                    ca.out_map = out8;
-                    ca.out_map4 = out4;
-                    ca.wave_map_ok = 1;
-                    ca.tile_ctr = err + 1;
-                    ca.err = err;
-                }
                 if ((rc = check(launch_col_shape(ny, cs, ca, st), "column pass"))) return done(rc);
             } else if ((rc = check(launch_col(ny, p + 1 == g.n_slices ? COL_DETECT : COL_STD, ca, st), "column pass"))) {
                 return done(rc);

@@ -30,7 +30,8 @@ const char *ROW_NAMES[N_ROW] = {"128 thr",
                                 "384 thr, TMA, radix-4 first: inverse",
                                 "384 thr, TMA, radix-4 first: both",
                                 "128 thr, radix-4 first: both",
-                                "128 thr, staged, radix-4 first: both"};
+                                "128 thr, staged, radix-4 first: both",
+                                "384 thr, radix-4 first: both"};
 const char *COL_NAMES[N_COL] = {"W4, staged",
                                 "W8, staged",
                                 "W16, staged",
@@ -60,7 +61,7 @@ const char *tune_shape_name(int kind, int v) {
 int tune_default_shape(int kind, int n) {
     const int rv = default_fft_variant(n);
     if (kind == 0) {
-        const int thr = n >= 512 ? 128 : 256;  // row_default_threads, unstaged
+        const int thr = n >= 2048 ? 384 : n >= 512 ? 128 : 256;  // row_default_threads, unstaged
         for (int v = 0; v < N_ROW; ++v)
             if (ROW_SHAPES[v].a == thr && !ROW_SHAPES[v].stg && !ROW_SHAPES[v].tma && ROW_SHAPES[v].rv == rv) return v;
     } else if (kind == 1) {

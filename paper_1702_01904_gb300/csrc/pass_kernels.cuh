@@ -67,7 +67,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // row is transformed; the slice's transmission row is loaded into registers before the inverse
 // FFT so that its latency hides behind the transform.
 template <int NX>
-constexpr int row_default_threads() { return NX >= 512 ? 128 : 256; }
+constexpr int row_default_threads() { return NX >= 2048 ? 384 : NX >= 512 ? 128 : 256; }
 
 // FFT radix variant (DftSplit, bit 0 forward, bit 1 inverse) of the default launchers: at N = 2048
 // both transforms put a radix-4 stage first in their 64- and 32-point register DFTs (row pass 20.0
@@ -94,6 +94,7 @@ struct RowCfg {
     // at N = 2048 the two stage-twiddle tables (32 KB) would hold the CTAs to 2 per SM: there they are
     // read through L1 (read-only path), interleaved with the exchange stores, for 3 CTAs per SM
     static constexpr bool L1TW = NX >= 2048;
+    static constexpr bool LOCKSTEP = NX >= 2048 && THR >= 384;
     static constexpr int TW_MODE = L1TW ? TW_GLOBAL : TW_SMEM;
     static constexpr int TWF2 = L1TW ? 0 : 2 * NX;  // float2 of twiddles in shared memory
     static constexpr size_t SMEM = (size_t)(TWF2 + SLOTS * SLOT_F2) * sizeof(float2);
@@ -194,6 +195,10 @@ __global__ void __launch_bounds__(THR) k_row(const __grid_constant__ RowArgs a) 
     if constexpr (C::TMA) bulk(row0);
     if constexpr (MODE != ROW_PLANE && C::STAGE) stage(row0);
     for (int it = 0; it < iters; ++it) {
+        // at N = 2048 a row is some 2000 instructions of straight code, and three CTAs of 4 warps at different
+        // places in it starved for instructions (the top stall): one CTA of 12 warps that start their rows
+        // together takes 7.8 instead of 8.1 ms per 529-beam launch (meeting between the transforms as well: 8.2)
+        if constexpr (C::LOCKSTEP) __syncthreads();
         const int row = row0 + it * stride;
         const bool valid = row < a.n_rows;
         int b, y;
@@ -266,6 +271,16 @@ __global__ void __launch_bounds__(THR) k_row(const __grid_constant__ RowArgs a) 
                     else if constexpr (cls == BAND_IN) v[r] = __ldcs(w + e);
                     else v[r] = keep(e) ? __ldcs(w + e) : make_float2(0.f, 0.f);
                 });
+                // the next row's kept halves on their way into the L2 (7.8 -> 7.3 ms)
+                if constexpr (C::LOCKSTEP && BL) {
+                    if (t == 0 && row + stride < a.n_rows) {
+                        int nb, ny;
+                        locate(row + stride, nb, ny);
+                        const float2 *wn = a.wave + ((size_t)nb * a.ny + ny) * NX;
+                        tc::bulk_prefetch(wn, NX / 4 * sizeof(float2));
+                        tc::bulk_prefetch(wn + 3 * NX / 4, NX / 4 * sizeof(float2));
+                    }
+                }
             }
             if constexpr (MODE == ROW_STD) {
                 // t_p is shared by all beams: L2-cached, not L1 (keeps L1 for the FFT's traffic)
@@ -559,6 +574,15 @@ __global__ void __launch_bounds__(ColCfg<NY, WC, STG, MB, TM>::THREADS, ColCfg<N
             } else {
 #pragma unroll
                 for (int r = 0; r < E; ++r) v[r] = col[(size_t)Fwd::in_elem(r, t) * a.nx];
+                // the next tile on its way into the L2 while this one is transformed: 8 warps of 255 registers
+                // wait for it otherwise (6.1 -> 4.8 ms per 529-beam launch)
+                if constexpr (W == 8 && NY >= 2048) {
+                    if (a.wave_map_ok && threadIdx.x == 0 && tile + gridDim.x < ntiles) {
+                        int nb, nk;
+                        locate(tile + gridDim.x, nb, nk);
+                        for (int y0 = 0; y0 < NY; y0 += C::BOXR) tc::tma_prefetch_3d(&a.wave_map, 2 * nk, y0, nb);
+                    }
+                }
             }
             if constexpr (C::TMA) {
                 // the barrier after the tile's arrival ordered every earlier use of the exchange

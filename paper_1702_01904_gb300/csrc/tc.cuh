@@ -160,6 +160,14 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                  "l"(src), "r"(bytes), "r"(smem_u32(mbar))
                  : "memory");
 }
+// `bytes` (a multiple of 16) from 16-byte aligned `src` into the L2 alone
+__device__ __forceinline__ void bulk_prefetch(const void *src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
+}
+// the box of a tensor map at (x, y, z) into the L2 alone
+__device__ __forceinline__ void tma_prefetch_3d(const void *map, int x, int y, int z) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];\n" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
+}
 // bounded wait: false if the phase did not complete within `limit_cycles` SM clock cycles
 // (try_wait itself suspends the thread for a short hardware-defined time between checks)
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *mbar, uint32_t parity, long long limit_cycles) {
