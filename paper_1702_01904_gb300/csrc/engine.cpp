@@ -391,6 +391,7 @@ struct prism_plan {
     CUtensorMap wave_map, wave_map4;  // the wave stack for the TMA-staged column pass (8 / 4 columns per box)
     CUtensorMap out_map, out_map4;    // its stores (ColArgs::out_map)
     bool shared_sms = false;   // a batch runs this plan's kernels beside other cells' (see col_default_shape)
+    bool scratch_budget = false;  // raster rows within the block scan's scratch (a batch over its budget)
     bool wave_map_ok = false;
     int *dev_err = nullptr;    // device error word
     int *col_ctr = nullptr;    // the TMA-staged column pass's tile counter and CTAs done (int[2])
@@ -940,6 +941,17 @@ extern "C" int prism_build_smatrix_host(prism_plan *P, const float *V_host) {
 }
 
 // ------------------------------------------------------------------ scan
+static int gemm_shape(const prism_plan *P);
+static int tc_shape(const prism_plan *P);
+// window scratch of the scan in blocks (0: kernels that need none)
+static size_t block_scratch(const prism_plan *P, int px, int py) {
+    if (P->prec == PRISM_PRECISION_FP32) {
+        const int sh = gemm_shape(P), grid = scan_gemm_grid(P->nw, P->nwy, sh, P->nbeams, px, py);
+        return grid > 0 ? scan_gemm_win_bytes(P->nw, P->nwy, sh, grid, px, py) : 0;
+    }
+    return scan_tc_win_bytes(P->nw, scan_tc_grid(P->nw, P->kp, tc_mode(P->prec), tc_shape(P), px, py), px, py);
+}
+
 // Whether the scan goes by raster rows (scan_rows.cuh), and its geometry: FP32 or FP16 value + remainder
 // S-matrix, every row of the raster on one y, rows of 3 probes or more, and few enough columns under the
 // rows' windows.  A row's sums cost one product per beam and column reached, then each probe one per
@@ -985,7 +997,9 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
     // 100 rows; 192 MB: 1.64 ms, 640 MB: 1.52)
     const size_t row = (size_t)P->nwy * planes * cols * sizeof(float2);
     const size_t blocks = ((size_t)sc->px + 3) / 4 * (((size_t)sc->py + 3) / 4);
-    const size_t most = std::min<size_t>(blocks, 304) * 64 * P->nw * P->nwy * sizeof(float2);
+    size_t most = std::min<size_t>(blocks, 304) * 64 * P->nw * P->nwy * sizeof(float2);
+    // (under a caller's tight budget no more than the blocks would take of this very scan)
+    if (P->scratch_budget) most = std::min(most, block_scratch(P, sc->px, sc->py));
     const size_t unpacked = split ? (size_t)P->nbeams * rows * cols * sizeof(float2) : 0;
     if (unpacked + row > most) return;
     const size_t limit = std::min<size_t>(most - unpacked, (size_t)384 << 20);
@@ -1214,15 +1228,15 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
     if (a.rows_lp > 0) {
         const size_t wb = (size_t)a.rows_chunk * P->nwy * (2 * a.rows_m + 1) * a.rows_cols * sizeof(float2);
         int rc = grow(P->arena, (void **)&P->rows_w, &P->rows_cap, wb);
-        if (rc) return rc;
-        a.rows_w = P->rows_w;
-        a.rows_src = P->S;
-        if (a.rows_unpack) {
-            if ((rc = grow(P->arena, (void **)&P->rows_s, &P->rows_s_cap, scan_rows_unpack_bytes(a)))) return rc;
-            a.rows_src = P->rows_s;
+        if (!rc && a.rows_unpack) rc = grow(P->arena, (void **)&P->rows_s, &P->rows_s_cap, scan_rows_unpack_bytes(a));
+        if (!rc) {
+            a.rows_w = P->rows_w;
+            a.rows_src = a.rows_unpack ? P->rows_s : P->S;
+            *grid = 1;
+            return PRISM_OK;
         }
-        *grid = 1;
-        return PRISM_OK;
+        cudaGetLastError();  // no memory for the rows: in blocks, whose scratch is smaller for long rasters
+        a.rows_lp = 0;
     }
     if (a.list) {
         *grid = 1;
@@ -2120,6 +2134,25 @@ extern "C" int prism_batch_create(const prism_cell *cells, int n_cells, size_t h
         const double px = (double)c.grid.nx * c.grid.ny;
         cost[i] = (double)P->nbeams * c.grid.n_slices * px * 32.0 +
                   (double)a.n_probes * P->nbeams * P->nw * P->nwy * (P->prec == PRISM_PRECISION_FP32 ? 8.0 : 1.0);
+    }
+    // over the budget with the scratch of the raster-row scans: again with no more than the block scans take
+    if (hbm_budget_bytes && bytes > hbm_budget_bytes) {
+        bytes = 0;
+        for (int i = 0; i < n_cells; ++i) {
+            prism_plan *P = B->plans[i];
+            ScanArgs &a = B->scans[i];
+            if (a.rows_lp > 0) {
+                P->scratch_budget = true;
+                if (P->rows_w) P->arena.forget(P->rows_w, P->rows_cap);
+                if (P->rows_s) P->arena.forget(P->rows_s, P->rows_s_cap);
+                P->rows_w = P->rows_s = nullptr;
+                P->rows_cap = P->rows_s_cap = 0;
+                if ((rc = scan_prepare(P, &cells[i].probe, &cells[i].scan, &cells[i].det, a, false)) || (rc = scan_setup(P, a, &B->scan_grid[i])))
+                    return fail(rc, "cell " + std::to_string(i) + ": " + g_err), bail(rc);
+                a.out = cells[i].out_dev;
+            }
+            bytes += P->arena.bytes;
+        }
     }
     if (hbm_budget_bytes && bytes > hbm_budget_bytes)
         return fail(PRISM_ERR_BUDGET, "batch needs " + std::to_string(bytes) + " bytes, budget " + std::to_string(hbm_budget_bytes)), bail(PRISM_ERR_BUDGET);

@@ -20,7 +20,7 @@
 //
 // Measured (40 000 probes of the 1024^2 carbon cell, 129 beams, 64-pixel windows): 5.03 ms with the
 // blocks of scan_gemm.cuh, 1.51 ms here (k_rows_sum 0.61, k_rows_window 0.84); 32 x 32 probes of the
-// 2048^2 cell (529 beams, 128-pixel windows) 2.68 -> 0.76 ms; 16 x 16 probes of a 256^2 cell 68 -> 33 us.
+// 2048^2 cell (529 beams, 128-pixel windows) 2.69 -> 0.76 ms; 16 x 16 probes of a 256^2 cell 68 -> 25 us.
 // 33 x 31 probes of a 512^2 cell from value + remainder storage (213 beams): 382 us on the tensor cores,
 // 110 us here, nearer to 64 bits (2.3e-6 against 4.9e-6 off).
 // Bound: k_rows_sum by the load/store pipe (67 % busy; its S reads hit the L2, 1.9 GB of them),
@@ -39,7 +39,9 @@
 
 namespace prism {
 
-constexpr int ROWS_R = 4;    // raster rows per k_rows_sum unit: each S value loaded feeds four sums
+// raster rows per k_rows_sum unit: each S value loaded feeds four sums (6 or 8 rows cost the registers and
+// shared memory of the third CTA per SM: 40 000 probes 1.50 ms with 4, 1.50 to 1.60 with 6, 1.70 with 8)
+constexpr int ROWS_R = 4;
 
 // ------------------------------------------------------------------ sums over n, column transforms
 // SMALL: for scans of few units, where a unit's latency counts and not the units an SM holds: more threads

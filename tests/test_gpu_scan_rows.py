@@ -2,13 +2,15 @@
 random values, at the edges of its tiles: windows of every size and shape, rows of 3 probes and of more
 than one CTA's, steps below a pixel and wider than a window, rows that wrap, run backwards or shift, and
 beam sets of one m up to several chunks of pairs."""
+import re
+
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
 from paper_1702_01904_gb300 import prism as P  # noqa: E402
-from paper_1702_01904_gb300.runtime import PrismSimulation  # noqa: E402
+from paper_1702_01904_gb300.runtime import Batch, PrismSimulation  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -121,6 +123,34 @@ def test_rows_of_value_and_remainder_storage(n, cell, f, alpha, kind, px, py, st
     cb = sim.scan_cbed(probe, x0, y0, px=px, py=py).cpu().numpy()
     close(cb, sim.scan_cbed(probe, x0, y0).cpu().numpy(), sim.info.n_beams, 2.0 ** -20)
     sim.close()
+
+
+@pytest.mark.parametrize("precision", [P.PRISM_PRECISION_FP32, P.PRISM_PRECISION_FP16X2])
+def test_batch_budget_bounds_the_rows_scratch(precision):
+    # a batch over its budget with the rows' scratch fits itself into that of the block scans (fewer rows at
+    # once, or blocks), with the results of the batch without a budget to rounding
+    n, cell = 256, 12.5
+    grid = P.make_grid(n, n, 1, cell, cell, 2.0, 300.0, 2, 2, 0.5, 28.0, precision=precision)
+    beams = PrismSimulation(grid).info.n_beams
+    V = 50.0 * torch.rand((1, n, n), generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+    x0, y0 = raster("plain", cell, 4, 41, 0.2)
+    c = dict(grid=grid, V=V, probe=P.make_probe(20.0), x0=x0, y0=y0, px=4, py=41, det=P.make_detector(0.0, 2.0, 40))
+    free = Batch([c])
+    free.run()
+    free.sync()
+    with pytest.raises(P.PrismError) as e:
+        Batch([c], hbm_budget_bytes=1)
+    least = int(re.search(r"batch needs (\d+) bytes", str(e.value)).group(1))
+    assert least < free.info.device_bytes
+    with pytest.raises(P.PrismError):
+        Batch([c], hbm_budget_bytes=least - 1)
+    tight = Batch([c], hbm_budget_bytes=least)
+    assert tight.info.device_bytes == least
+    tight.run()
+    tight.sync()
+    close(tight.outs[0].cpu().numpy(), free.outs[0].cpu().numpy().astype(np.float64), beams, 2.0 ** -20)
+    free.close()
+    tight.close()
 
 
 @pytest.mark.parametrize("n,cell,f,f_y,alpha", [(64, 8.0, 2, 0, 20.0), (64, 8.0, 2, 1, 20.0), (128, 12.8, 1, 4, 20.0), (256, 16.0, 4, 0, 20.0),
