@@ -484,6 +484,7 @@ def main():
     with torch.cuda.stream(stream):
         sim = PrismSimulation(grid, 0, stream)
         Bn = sim.info.n_beams
+        beam_m = [int(m) for m in sim.beams()[0]]
         tune = None if args.no_autotune else sim.autotune(fft_radix=True)
         out = torch.empty((P, DET["nbins"]), dtype=torch.float32, device="cuda")
 
@@ -684,7 +685,7 @@ def main():
                 tf = fft_flops[name] / (r["mean_ms"] / 1000.0) / 1e12
                 roof_all[name].update({"fft_tflops": tf, "fft_peak_tflops": fp32_peak, "fft_frac": tf / fp32_peak,
                                        "fft_flops_per_launch": fft_flops[name]})
-        elif name == "scan" and args.precision != "fp32":
+        elif name == "scan" and args.precision not in ("fp32", "fp16x2"):
             # beam sum on the tensor cores: 8 real flops per complex MAC, against the measured dense
             # 16-bit rate (sustained: the scan runs inside a seconds-long loop of steps)
             nw = w.nx // w.downsample // w.f
@@ -694,9 +695,13 @@ def main():
             roof_all[name] = {"bound": "tensor", "achieved": tf, "peak": peak_tf, "unit": "TFLOP/s",
                               "frac": tf / peak_tf, "flops_per_launch": flops, **r}
         elif name == "scan":
-            # ALU-bound: 8 flops per complex MAC of the beam sum (a7) + window FFTs
-            nw = w.nx // w.downsample // w.f
-            flops = P * (8.0 * Bn * nw * nw + 2 * 5.0 * nw * nw * math.log2(nw))
+            # the sum separated on raster rows: 8 flops per complex MAC of a row's beams over the columns
+            # its windows reach, the column transforms of its 2 M + 1 planes there, then per probe 8 flops
+            # per pair +-m and pixel (two real-by-complex products) and the row transforms
+            nw, n_m = w.nx // w.downsample // w.f, len(set(beam_m))
+            cols = min(w.nx // w.downsample, nw + (w.scan_px - 1) * w.scan_step * w.nx / (w.downsample * w.cell_x))
+            flops = (w.scan_py * cols * (8.0 * Bn * nw + n_m * fl(nw)) +
+                     P * nw * (4.0 * (n_m - 1) * nw + 2.0 * nw + fl(nw)))
             clk_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
             peak_tf = 152 * 128 * 2 * clk_mhz * 1e6 / 1e12
             tf = flops / (r["mean_ms"] / 1000.0) / 1e12
