@@ -20,7 +20,7 @@
 //
 // Measured (40 000 probes of the 1024^2 carbon cell, 129 beams, 64-pixel windows): 5.03 ms with the
 // blocks of scan_gemm.cuh, 1.51 ms here (k_rows_sum 0.61, k_rows_window 0.84); 32 x 32 probes of the
-// 2048^2 cell (529 beams, 128-pixel windows) 2.69 -> 0.76 ms; 16 x 16 probes of a 256^2 cell 68 -> 25 us.
+// 2048^2 cell (529 beams, 128-pixel windows) 2.70 -> 0.73 ms; 16 x 16 probes of a 256^2 cell 68 -> 25 us.
 // 33 x 31 probes of a 512^2 cell from value + remainder storage (213 beams): 382 us on the tensor cores,
 // 110 us here, nearer to 64 bits (2.3e-6 against 4.9e-6 off).
 // Bound: k_rows_sum by the load/store pipe (67 % busy; its S reads hit the L2, 1.9 GB of them),
@@ -49,12 +49,16 @@ constexpr int ROWS_R = 4;
 template <int NWY, bool SMALL = false>
 struct RowsSumCfg {
     using FS = FftShape<NWY>;
-    static constexpr int BLOCK = SMALL ? 256 : 192;
-    static constexpr int MINB = SMALL ? 1 : 3;
-    static constexpr int XC = NWY >= 128 ? 8 : 16;       // columns per unit: 64- or 128-byte runs of S and of W
+    // 128-pixel windows: the columns' buffers (79 KB) leave two CTAs on an SM anyway, so they take more threads and
+    // loads in flight (529 beams, 32 x 32 probes, whole scan: 762 us with 192 threads and 7 loads, 765 with 288
+    // and 7, 731 with 192 and 14, 717 with 288 and 9, 714 so)
+    static constexpr bool WIDE = NWY >= 128;
+    static constexpr int BLOCK = SMALL || WIDE ? 256 : 192;
+    static constexpr int MINB = SMALL ? 1 : WIDE ? 2 : 3;
+    static constexpr int XC = WIDE ? 8 : 16;             // columns per unit: 64- or 128-byte runs of S and of W
     static constexpr int PAIRS = XC / 2;                 // a thread takes two neighbouring columns
     static constexpr int YSTEP = BLOCK / PAIRS;          // union rows per sweep of the block
-    static constexpr int U = SMALL ? 14 : 7;             // beams whose loads a thread issues together
+    static constexpr int U = SMALL ? 14 : WIDE ? 13 : 7; // beams whose loads a thread issues together
     // A column of one plane and raster row: NWY values, in place the transform's exchange.  The second
     // column of a pair starts 16 banks on (mod 32), so the columns two slots of a half-warp transform
     // fall on different banks; pairs are 4 banks apart (8 for the 4 pairs of 8 columns), so that the
