@@ -502,6 +502,16 @@ int prism_plan_set_profiling(prism_plan *plan, int enable);
 int prism_plan_kernel_stats(prism_plan *plan, int kind, long *launches, double *total_ms);
 /* Total kernel launches issued by the plan since creation (or the last reset). */
 long prism_plan_launches(const prism_plan *plan);
+/* The kernels that the plan's last scan took (PRISM_SCAN_*): by raster rows, probe by probe, in blocks
+ * of 32 probes on the CUDA cores or on the tensor cores, or the kernels of windows and beam sets that fit
+ * none of these. */
+int prism_plan_scan_path(const prism_plan *plan);
+#define PRISM_SCAN_NONE 0
+#define PRISM_SCAN_ROWS 1
+#define PRISM_SCAN_LIST 2
+#define PRISM_SCAN_BLOCKS 3
+#define PRISM_SCAN_TENSOR 4
+#define PRISM_SCAN_OTHER 5
 int prism_plan_reset_stats(prism_plan *plan);
 const char *prism_kernel_name(int kind);
 

@@ -442,6 +442,7 @@ struct prism_plan {
     int det_nbins = -1;
     // statistics
     long launches = 0;
+    int scan_path = PRISM_SCAN_NONE;  // of the last scan
     bool profiling = false;
     std::vector<PendingEv> pending;
     std::vector<cudaEvent_t> ev_pool;
@@ -1263,6 +1264,11 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
 }
 
 static int scan_go(prism_plan *P, const ScanArgs &a, int grid) {
+    P->scan_path = a.rows_lp > 0                          ? PRISM_SCAN_ROWS
+                   : a.list                               ? PRISM_SCAN_LIST
+                   : P->prec != PRISM_PRECISION_FP32      ? PRISM_SCAN_TENSOR
+                   : grid > 0                             ? PRISM_SCAN_BLOCKS
+                                                          : PRISM_SCAN_OTHER;
     if (a.rows_lp > 0) {
         const int rc = plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_rows(P->nw, P->nwy, a, P->stream); });
         P->rows_attrs = P->rows_attrs || !rc;
@@ -1720,6 +1726,7 @@ extern "C" int prism_plan_kernel_stats(prism_plan *P, int kind, long *launches, 
 }
 
 extern "C" long prism_plan_launches(const prism_plan *P) { return P ? P->launches : 0; }
+extern "C" int prism_plan_scan_path(const prism_plan *P) { return P ? P->scan_path : PRISM_SCAN_NONE; }
 
 extern "C" int prism_plan_reset_stats(prism_plan *P) {
     if (!P) return fail(PRISM_ERR_INVALID, "plan is NULL");

@@ -41,6 +41,9 @@ PRISM_BATCH_AUTOTUNE = 1
 PRISM_BATCH_AUTOTUNE_FFT_RADIX = 2
 PRISM_AUTOTUNE_FFT_RADIX = 1
 
+# which kernels a plan's last scan took (prism_plan_scan_path)
+PRISM_SCAN_NONE, PRISM_SCAN_ROWS, PRISM_SCAN_LIST, PRISM_SCAN_BLOCKS, PRISM_SCAN_TENSOR, PRISM_SCAN_OTHER = range(6)
+
 # every entry point declared in include/prism.h
 EXPORTED = [
     "prism_plan_create", "prism_plan_destroy", "prism_sync", "prism_last_error",
@@ -48,7 +51,7 @@ EXPORTED = [
     "prism_scan_run_cbed", "prism_scan_run_accumulate",
     "multislice_scan_run", "multislice_scan_run_noalloc", "prism_plan_info", "prism_plan_smatrix_bytes", "prism_plan_beams",
     "prism_plan_smatrix", "prism_plan_smatrix_copy", "prism_plan_transmission", "prism_wavelength", "prism_interaction_constant",
-    "prism_recommended_alpha_max", "prism_plan_set_profiling", "prism_plan_kernel_stats", "prism_plan_launches", "prism_plan_reset_stats",
+    "prism_recommended_alpha_max", "prism_plan_set_profiling", "prism_plan_kernel_stats", "prism_plan_launches", "prism_plan_scan_path", "prism_plan_reset_stats",
     "prism_kernel_name",
     "prism_server_create", "prism_server_submit", "prism_server_wait", "prism_server_stats", "prism_server_destroy",
     "prism_server_cancel",
@@ -175,6 +178,7 @@ def load(path: str = LIB_PATH):
         "prism_plan_set_profiling": (c_int, [P, c_int]),
         "prism_plan_kernel_stats": (c_int, [P, c_int, POINTER(c_long), POINTER(c_double)]),
         "prism_plan_launches": (c_long, [P]),
+        "prism_plan_scan_path": (c_int, [P]),
         "prism_plan_reset_stats": (c_int, [P]),
         "prism_kernel_name": (c_char_p, [c_int]),
         "prism_server_create": (c_int, [c_size_t, c_int, POINTER(P)]),
@@ -383,6 +387,10 @@ def prism_plan_kernel_stats(plan, kind):
 
 def prism_plan_launches(plan):
     return load().prism_plan_launches(plan)
+
+
+def prism_plan_scan_path(plan):
+    return load().prism_plan_scan_path(plan)
 
 
 def prism_plan_reset_stats(plan):

@@ -1,0 +1,168 @@
+"""Every kernel that a scan can take, with the path asserted: the block scan's contraction shapes, split blocks,
+work-unit counters, scratch and shared-memory limits on positions that go by blocks (rasters of many probes
+whose rows do not share a y, tall rasters of two columns)."""
+import threading
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1702_01904_gb300 import prism as P  # noqa: E402
+from paper_1702_01904_gb300.runtime import PrismSimulation  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+DET = P.make_detector(0.0, 2.0, 40)
+PROBE = P.make_probe(20.0, 12.0)
+
+
+def plan(n, cell, f, seed, f_y=0, alpha=20.0, precision=P.PRISM_PRECISION_FP32):
+    sim = PrismSimulation(P.make_grid(n, n, 1, cell, cell, 2.0, 300.0, f, 2, 0.5, alpha, f_y=f_y, precision=precision))
+    i = sim.info
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    sim.load_smatrix(torch.view_as_complex(torch.randn((i.n_beams, i.ny_s, i.nx_s, 2), generator=g, device="cuda")))
+    return sim
+
+
+def jittered(px, py, step, seed=0):
+    # a raster whose probes are off their row by up to a quarter of a step, across the cell's edges
+    r = np.random.default_rng(seed)
+    x, y = np.meshgrid(step * np.arange(px) - 1.3, step * np.arange(py) - 0.7)
+    return x.ravel(), (y + 0.25 * step * r.uniform(-1.0, 1.0, y.shape)).ravel()
+
+
+def scan(sim, pos, px, py, path):
+    out = sim.scan(PROBE, *pos, DET, px=px, py=py).cpu().numpy()
+    assert P.prism_plan_scan_path(sim.plan) == path
+    return out
+
+
+def exact(sim, cell, f, f_y, x0, y0):
+    """Bins of the probes in 64 bits."""
+    i = sim.info
+    m, k = sim.beams()
+    f_y = f_y or f
+    lam = P.prism_wavelength(300.0)
+    qx, qy = m * f / cell, k * f_y / cell
+    inside = (lam * qx) ** 2 + (lam * qy) ** 2 <= 0.02 ** 2 * (1 + 1e-12)
+    A = inside * np.exp(-1j * np.pi * lam * (qx ** 2 + qy ** 2) * 12.0)
+    S = sim.smatrix().cpu().numpy().astype(np.complex128)
+    wx, wy = (np.fft.fftfreq(n, 1.0 / n) * ff / cell for n, ff in ((i.nw_x, f), (i.nw_y, f_y)))
+    b = np.floor(1000.0 * lam * np.sqrt(wx[None, :] ** 2 + wy[:, None] ** 2) / 2.0).astype(int)
+    out = []
+    for x, y in zip(x0, y0):
+        a = A * np.exp(-2j * np.pi * (qx * x + qy * y))
+        ix = (int(np.floor(x / (cell / i.nx_s) + 0.5)) - i.nw_x // 2 + np.arange(i.nw_x)) % i.nx_s
+        iy = (int(np.floor(y / (cell / i.ny_s) + 0.5)) - i.nw_y // 2 + np.arange(i.nw_y)) % i.ny_s
+        psi = np.tensordot(a, S[:, iy[:, None], ix[None, :]], axes=(0, 0))
+        inten = np.abs(np.fft.fft2(psi)) ** 2 / ((i.nw_x * i.nw_y) ** 2 * inside.sum())
+        out.append([inten[b == j].sum() for j in range(40)])
+    return np.array(out)
+
+
+def close(got, ref, beams):
+    # one rounding of 2^-24 per beam, butterfly stage and combination at most, an FP32 coefficient of 2^-22
+    # per product besides, twice that for intensities
+    err = np.linalg.norm(got.astype(np.float64) - ref) / np.linalg.norm(ref)
+    assert err <= 2.0 * ((beams + 24) * 2.0 ** -24 + 2.0 ** -22 * beams ** 0.5), err
+
+
+# windows of 16, 32 and 64 pixels; sides that leave partial blocks of 4 x 8, 8 x 4 and 2 x 16
+@pytest.mark.parametrize("n,cell,f,px,py,step", [(128, 8.0, 4, 101, 97, 0.11), (128, 12.8, 2, 53, 49, 0.2), (512, 32.0, 4, 47, 45, 0.1)])
+def test_block_scan_in_every_contraction_shape(n, cell, f, px, py, step):
+    sim = plan(n, cell, f, 1)
+    pos = jittered(px, py, step)
+    ref = scan(sim, pos, px, py, P.PRISM_SCAN_BLOCKS)
+    some = np.array([0, px - 1, 7 * px + 5, px * py // 2, px * py - 1])
+    close(ref[some], exact(sim, cell, f, 0, pos[0][some], pos[1][some]), sim.info.n_beams)
+    shapes = P.prism_plan_tune_result(sim.plan, P.PRISM_TUNE_SCAN).n_shapes
+    assert shapes == 6
+    for v in range(shapes):
+        sim.set_shape(P.PRISM_TUNE_SCAN, v)
+        assert np.array_equal(scan(sim, pos, px, py, P.PRISM_SCAN_BLOCKS), ref), P.prism_tune_shape_name(P.PRISM_TUNE_SCAN, v)
+    sim.set_shape(P.PRISM_TUNE_SCAN, -1)
+    out = sim.autotune_scan(PROBE, *pos, DET, px=px, py=py).cpu().numpy()
+    assert P.prism_plan_scan_path(sim.plan) == P.PRISM_SCAN_BLOCKS and np.array_equal(out, ref)
+    ms = sim.tune_result()["scan"]["ms"]
+    assert len(set(ms.values())) > 1 and ms[sim.tune_result()["scan"]["chosen"]] == min(ms.values())
+    sim.close()
+
+
+@pytest.mark.parametrize("f,f_y", [(8, 4), (4, 8), (4, 2)])
+def test_block_scan_of_unequal_windows(f, f_y):
+    # 16 x 32, 32 x 16 and 32 x 64 pixels
+    sim = plan(256, 16.0, f, 2, f_y=f_y)
+    px, py = 83, 90
+    pos = jittered(px, py, 0.13)
+    out = scan(sim, pos, px, py, P.PRISM_SCAN_BLOCKS)
+    some = np.array([0, px - 1, px * py - 1])
+    close(out[some], exact(sim, 16.0, f, f_y, pos[0][some], pos[1][some]), sim.info.n_beams)
+    sim.close()
+
+
+@pytest.mark.parametrize("shape", range(6))
+def test_block_scan_grows_its_scratch_for_each_shape(shape):
+    # a small first scan by blocks, then a pinned shape and a larger raster
+    n, cell, f = 128, 12.8, 2
+    small, pos = jittered(40, 52, 0.2, 3), jittered(101, 99, 0.1, 4)
+    sim = plan(n, cell, f, 3)
+    ref = scan(sim, pos, 101, 99, P.PRISM_SCAN_BLOCKS)
+    sim.close()
+    sim = plan(n, cell, f, 3)
+    scan(sim, small, 40, 52, P.PRISM_SCAN_BLOCKS)
+    sim.set_shape(P.PRISM_TUNE_SCAN, shape)
+    assert np.array_equal(scan(sim, pos, 101, 99, P.PRISM_SCAN_BLOCKS), ref)
+    sim.close()
+
+
+def test_block_scan_bands_and_repeats_bitwise():
+    # 320 blocks of 4 x 8 (more than the CTAs: the last round is split) against bands of 16 rows (80 blocks,
+    # all split), on one plan in turn: the split changes no bit and the work-unit counters, whose place moves
+    # with the grid, are left zero
+    sim = plan(128, 12.8, 2, 5)
+    pos = jittered(160, 64, 0.09, 5)
+    whole = scan(sim, pos, 160, 64, P.PRISM_SCAN_BLOCKS)
+    for r in range(0, 64, 16):
+        e = slice(r * 160, (r + 16) * 160)
+        band = scan(sim, (pos[0][e], pos[1][e]), 160, 16, P.PRISM_SCAN_BLOCKS)
+        assert np.array_equal(band, whole[e])
+        assert np.array_equal(scan(sim, pos, 160, 64, P.PRISM_SCAN_BLOCKS), whole)
+    sim.close()
+
+
+def test_block_scan_of_two_columns():
+    x, y = np.meshgrid(0.2 + 0.2 * np.arange(2), 0.05 * np.arange(1040))
+    sim = plan(128, 12.8, 2, 6)
+    out = scan(sim, (x.ravel(), y.ravel()), 2, 1040, P.PRISM_SCAN_BLOCKS)
+    some = np.array([0, 1, 1039, 2079])
+    close(out[some], exact(sim, 12.8, 2, 0, x.ravel()[some], y.ravel()[some]), sim.info.n_beams)
+    sim.close()
+
+
+def test_block_scans_of_different_beam_counts_at_once():
+    # the shared-memory limit of one kernel, from four threads with plans of different beam counts
+    sims = [plan(256, 16.0, 4, 7 + i, alpha=a) for i, a in enumerate((20.0, 15.0, 28.0, 18.0))]
+    assert len({s.info.n_beams for s in sims}) == 4
+    pos = jittered(65, 63, 0.2, 7)
+    refs = [scan(s, pos, 65, 63, P.PRISM_SCAN_BLOCKS) for s in sims]
+    outs, errors = [None] * 4, []
+
+    def worker(i):
+        try:
+            for _ in range(5):
+                o = sims[i].scan(PROBE, *pos, DET, px=65, py=63)
+                sims[i].sync()
+            outs[i] = o.cpu().numpy()
+        except Exception as e:  # reported below
+            errors.append(e)
+
+    threads = [threading.Thread(target=worker, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join(timeout=300)
+    assert not errors, errors
+    for s, o, r in zip(sims, outs, refs):
+        assert np.array_equal(o, r)
+        s.close()
