@@ -140,19 +140,34 @@ __global__ void __launch_bounds__(ListCfg<NWX, NWY>::BLOCK) k_scan_list(const __
         }
     }
     if (!a.out) return;
-    // a warp per annular bin: lanes over its pixel list, FP32 partial sums, a fixed xor tree, FP64 scale
-    const int lane = tid & 31;
-    for (int k = tid >> 5; k < a.nbins; k += BLOCK / 32) {
-        float s = 0.f;
-        const int e = __ldg(a.bin_off + k + 1);
-        for (int i = __ldg(a.bin_off + k) + lane; i < e; i += 32) {
-            const int u = __ldg(a.bin_idx + i);
-            const float2 z = win[(u >> LNW) * PW + (u & (NWX - 1))];
-            s = fmaf(z.x, z.x, fmaf(z.y, z.y, s));
+    // a warp per annular bin: lanes over its pixel list, their FP32 sums folded to four (of the entries i mod 4;
+    // no more additions deep than the four of window_outputs), which one lane per bin adds and scales in
+    // FP64, 32 bins at a time
+    constexpr int WARPS = BLOCK / 32;
+    const int lane = tid & 31, warp = tid >> 5;
+#pragma unroll 1
+    for (int k0 = warp; k0 < a.nbins; k0 += 32 * WARPS) {
+        float4 part = make_float4(0.f, 0.f, 0.f, 0.f);  // of bin k0 + WARPS lane
+#pragma unroll 1
+        for (int j = 0; j < 32; ++j) {
+            const int k = k0 + WARPS * j;
+            if (k >= a.nbins) break;
+            float s = 0.f;
+            const int e = __ldg(a.bin_off + k + 1);
+            for (int i = __ldg(a.bin_off + k) + lane; i < e; i += 32) {
+                const int u = __ldg(a.bin_idx + i);
+                const float2 z = win[(u >> LNW) * PW + (u & (NWX - 1))];
+                s = fmaf(z.x, z.x, fmaf(z.y, z.y, s));
+            }
+#pragma unroll
+            for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            const float4 q = make_float4(__shfl_sync(0xffffffffu, s, 0), __shfl_sync(0xffffffffu, s, 1), __shfl_sync(0xffffffffu, s, 2),
+                                         __shfl_sync(0xffffffffu, s, 3));
+            if (lane == j) part = q;
         }
-        s = warp_sum(s);
-        if (lane == 0) {
-            const float val = (float)((double)s * a.inv_norm);
+        const int k = k0 + WARPS * lane;
+        if (k < a.nbins) {
+            const float val = (float)((((double)part.x + (double)part.y) + ((double)part.z + (double)part.w)) * a.inv_norm);
             float *o = a.out + (size_t)p * a.nbins + k;
             *o = a.accumulate ? *o + a.acc_w * val : val;
         }

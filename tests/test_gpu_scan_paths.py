@@ -166,3 +166,26 @@ def test_block_scans_of_different_beam_counts_at_once():
     for s, o, r in zip(sims, outs, refs):
         assert np.array_equal(o, r)
         s.close()
+
+
+def test_list_bins_are_added_in_64_bits():
+    # the bins of scattered probes with 64-pixel windows against FP64 sums of their diffraction patterns: one beam
+    # in the aperture, so that the normalisation 2^-24 is exact.  A bin of at most 32 pixels is four FP32 sums
+    # of three additions' depth, added in FP64 and rounded: (1 + 1/2 + 1/4) / 4 + 1 roundings' variance, 1.2 rms,
+    # and the patterns' own add little; five additions deep in FP32 and then rounded it would be 1.71.  Half way
+    # between: 1.45, a rounding of 2^-24 being 0.425 rms (uniform, mantissas spread over their logarithm).
+    sim = plan(512, 32.0, 4, 8)
+    i = sim.info
+    r = np.random.default_rng(8)
+    pos = (r.uniform(0.0, 32.0, 400), r.uniform(0.0, 32.0, 400))
+    probe = P.make_probe(1.0)
+    inten = sim.scan_cbed(probe, *pos).cpu().numpy().reshape(400, -1).astype(np.float64)
+    assert P.prism_plan_scan_path(sim.plan) == P.PRISM_SCAN_LIST
+    out = sim.scan(probe, *pos, P.make_detector(0.0, 1.0, 100)).cpu().numpy()
+    assert P.prism_plan_scan_path(sim.plan) == P.PRISM_SCAN_LIST
+    w = np.fft.fftfreq(i.nw_x, 1.0 / i.nw_x) * 4 / 32.0
+    b = np.floor(1000.0 * i.wavelength * np.sqrt(w[None, :] ** 2 + w[:, None] ** 2)).astype(int).ravel()
+    err = np.concatenate([out[:, k] / inten[:, b == k].sum(1) - 1.0 for k in range(100) if 12 <= (b == k).sum() <= 32])
+    assert err.size > 5000
+    assert np.sqrt(np.mean(err ** 2)) <= 1.45 * 0.425 * 2.0 ** -24
+    sim.close()
