@@ -64,9 +64,19 @@ __global__ void __launch_bounds__(ListCfg<NWX, NWY>::BLOCK) k_scan_list(const __
     const int wx = tid % NWX, wy = tid / NWX;  // this thread's pixels: column wx, rows wy + RS k
     const float2 *Sx = a.S + ((sx + wx) & (a.nx_s - 1));
     const size_t bstride = (size_t)a.ny_s * a.nx_s;
-    float2 acc[PIX];
+    // Up to 8 pixels: the two sums of scan_gemm.cuh, sum_b S_b Re alpha_b and sum_b S_b Im alpha_b, advanced
+    // by one packed FMA each: the same windows bit by bit.  More: the registers hold one sum, rounded twice per
+    // beam by its two FMAs, so every 16 beams it goes to the window in shared memory (400 probes of 213 beams,
+    // bins against 64 bits: 1.2e-7 off in one chain, 0.95e-7 by two sums, 0.80e-7 so; 0.46 -> 0.48 ms for 900.
+    // Two sums with half the loads in flight: 0.63 ms)
+    constexpr bool TWO = PIX <= 8;
+    constexpr int RUN = 16;
+    float2 acc[PIX], aci[TWO ? PIX : 1];
 #pragma unroll
     for (int k = 0; k < PIX; ++k) acc[k] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < (TWO ? PIX : 1); ++k) aci[k] = make_float2(0.f, 0.f);
+    auto out = [&](int k) -> float2 & { return win[(wy + RS * k) * PW + wx]; };
     __syncthreads();
     constexpr int PB = C::PB, NB = C::NB;
     auto load = [&](float2 (&s)[U][PB], int b0, int h) {  // batch h of beams b0 ... b0 + U - 1
@@ -92,10 +102,15 @@ __global__ void __launch_bounds__(ListCfg<NWX, NWY>::BLOCK) k_scan_list(const __
                     const float2 al = alpha[b0 + i];
 #pragma unroll
                     for (int k = 0; k < PB; ++k) {
-                        float2 &c = acc[h * PB + k];
                         const float2 s = cur[i][k];
-                        c.x = fmaf(al.x, s.x, fmaf(-al.y, s.y, c.x));
-                        c.y = fmaf(al.x, s.y, fmaf(al.y, s.x, c.y));
+                        if constexpr (TWO) {
+                            acc[h * PB + k] = __ffma2_rn(s, make_float2(al.x, al.x), acc[h * PB + k]);
+                            aci[h * PB + k] = __ffma2_rn(s, make_float2(al.y, al.y), aci[h * PB + k]);
+                        } else {
+                            float2 &c = acc[h * PB + k];
+                            c.x = fmaf(al.x, s.x, fmaf(-al.y, s.y, c.x));
+                            c.y = fmaf(al.x, s.y, fmaf(al.y, s.x, c.y));
+                        }
                     }
                 }
 #pragma unroll
@@ -103,20 +118,35 @@ __global__ void __launch_bounds__(ListCfg<NWX, NWY>::BLOCK) k_scan_list(const __
 #pragma unroll
                 for (int k = 0; k < PB; ++k) cur[i][k] = nxt[i][k];
         }
-    }
+        if constexpr (!TWO) {
+            static_assert(TWO || U == 1, "a beam per step");
+            const int done = b0 - bb + 1;
+            if (done % RUN == 0 || b0 + 1 == be) {
 #pragma unroll
-    for (int k = 0; k < PIX; ++k) win[(wy + RS * k) * PW + wx] = acc[k];
+                for (int k = 0; k < PIX; ++k) {
+                    out(k) = done <= RUN ? acc[k] : cadd(out(k), acc[k]);
+                    acc[k] = make_float2(0.f, 0.f);
+                }
+            }
+        }
+    }
+    if (TWO || bb == be) {
+#pragma unroll
+        for (int k = 0; k < PIX; ++k) out(k) = TWO ? make_float2(acc[k].x - aci[TWO ? k : 0].y, acc[k].y + aci[TWO ? k : 0].x) : acc[k];
+    }
     if (cn > 1) {
         // every rank's window is written; the first adds the others' to its own, then they may leave
         cl.sync();
         if (cr == 0) {
+#pragma unroll
+            for (int k = 0; k < PIX; ++k) acc[k] = out(k);
             for (int r = 1; r < cn; ++r) {
                 const float2 *o = cl.map_shared_rank(win, r);
 #pragma unroll
                 for (int k = 0; k < PIX; ++k) acc[k] = cadd(acc[k], o[(wy + RS * k) * PW + wx]);
             }
 #pragma unroll
-            for (int k = 0; k < PIX; ++k) win[(wy + RS * k) * PW + wx] = acc[k];
+            for (int k = 0; k < PIX; ++k) out(k) = acc[k];
         }
         cl.sync();
         if (cr != 0) return;

@@ -189,3 +189,43 @@ def test_list_bins_are_added_in_64_bits():
     assert err.size > 5000
     assert np.sqrt(np.mean(err ** 2)) <= 1.45 * 0.425 * 2.0 ** -24
     sim.close()
+
+
+@pytest.mark.parametrize("n,cell,f,f_y", [(128, 8.0, 4, 0), (128, 12.8, 2, 0), (256, 16.0, 8, 4), (256, 16.0, 4, 8)])
+def test_list_equals_blocks_bitwise(n, cell, f, f_y):
+    # windows of up to 1024 pixels: probes from a raster that goes by blocks, scanned as a list (long enough that
+    # no two CTAs share a probe's beams)
+    sim = plan(n, cell, f, 9, f_y=f_y)
+    pos = jittered(101, 97, 0.11, 9)
+    whole = scan(sim, pos, 101, 97, P.PRISM_SCAN_BLOCKS)
+    some = np.random.default_rng(9).choice(101 * 97, 300, replace=False)
+    part = scan(sim, (pos[0][some], pos[1][some]), 300, 1, P.PRISM_SCAN_LIST)
+    assert np.array_equal(part, whole[some])
+    sim.close()
+
+
+def test_list_sums_over_beams():
+    # 64-pixel windows, 213 beams of independent random values: no further from 64 bits than the block scan's two
+    # sums.  Each of those is rounded once per beam at a size growing as the root of the beams summed: B / 2
+    # roundings' variance against the whole, a rounding of 2^-24 being 0.425 rms; 20 more for the coefficients
+    # and two transforms of 6 stages.  One chain rounded twice per beam has B of them.
+    sim = plan(512, 32.0, 4, 10)
+    i = sim.info
+    r = np.random.default_rng(10)
+    x, y = r.uniform(0.0, 32.0, 300), r.uniform(0.0, 32.0, 300)  # (long enough that no two CTAs share a probe's beams)
+    out = sim.scan_cbed(P.make_probe(20.0), x, y).cpu().numpy()
+    assert P.prism_plan_scan_path(sim.plan) == P.PRISM_SCAN_LIST
+    m, k = sim.beams()
+    qx, qy = m * 4 / 32.0, k * 4 / 32.0
+    S = sim.smatrix().cpu().numpy().astype(np.complex128)
+    num = den = 0.0
+    for p in range(0, 300, 10):
+        a = np.exp(-2j * np.pi * (qx * x[p] + qy * y[p]))
+        ix = (int(np.floor(x[p] / 0.125 + 0.5)) - 32 + np.arange(64)) % 256
+        iy = (int(np.floor(y[p] / 0.125 + 0.5)) - 32 + np.arange(64)) % 256
+        ref = np.abs(np.fft.fft2(np.tensordot(a, S[:, iy[:, None], ix[None, :]], axes=(0, 0)))) ** 2 / (4096.0 ** 2 * len(m))
+        num += np.sum((out[p] - ref) ** 2)
+        den += np.sum(ref ** 2)
+    assert i.n_beams == len(m) == 213
+    assert np.sqrt(num / den) <= 0.425 * 2.0 ** -24 * np.sqrt(213 / 2 + 20)
+    sim.close()
