@@ -1030,37 +1030,53 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
 // Whether the scan goes probe by probe (scan_list.cuh): FP32, not by raster rows, and
 //  - at least half of the 4 x 8 blocks of the general scan (scan_gemm.cuh) could not share a union tile (its
 //    test, by the extent of their positions: larger in pixels than their windows together), or
-//  - the raster does not fill blocks (fewer than 8 rows of it: a list of positions fills 4 slots of a
-//    block's 32), or has fewer than 2048 probes; of 128-pixel windows fewer than 64.
-// Measured, blocks against probe by probe: 900 scattered probes 1.32 -> 0.34 ms (129 beams, 64-pixel windows),
-// 2.80 -> 0.47 (213), 10 of them 317 -> 35 us; a dense line of 900 0.45 -> 0.33; a rotated 30 x 30 raster
-// 0.38 -> 0.26, but 63 x 63 0.86 -> 1.13; 128-pixel windows: 10 probes 0.42 -> 0.23, 100 on a line
-// 0.92 -> 1.39, 900 scattered 24.9 -> 14.7.
+//  - by the estimates below it takes less than 0.95 of the time in blocks.
+// Probe by probe: 19 us of launch and host, 2.5e-3 us per probe, 7.7e-6 per window pixel (transform, bins) and
+// 4.3e-7 per beam and window pixel (64-pixel windows 6.5e-7, and 1e-6 where the S values under them, 80 MB or
+// more, outgrow the L2's nearer part).  Blocks: a round of 304 (one per resident CTA) takes 19 us, 1e-3 us per beam and pixel of the union
+// tile, less where blocks are split over idle CTAs, and 1.33e-3 us per window pixel of its 32 probes.  The
+// constants are a fit to 1900 scans (windows of 16 to 64 pixels, 9 to 405 beams, rasters of 1 x 1 to 120 x 120
+// turned or jittered, steps of 0.05 to 3 A), both ways measured; with them no scan was slower than in blocks by
+// more than the runs differ.  (A bound of 2048 probes, whatever the beams, had 1600 turned probes of 213 beams and
+// 64-pixel windows take 694 us instead of 435.)  128-pixel windows: fewer than 64 probes, 8000 beams of
+// probes (10 of 529 beams 0.42 -> 0.23 ms, 36 of them on a line 0.45 -> 0.69; 60 of 109 beams 0.67 -> 0.14).
+// 16 blocks spread over the raster stand for all.
 static void position_list(const prism_plan *P, const prism_scan *sc, ScanArgs &a) {
-    if (P->prec != PRISM_PRECISION_FP32 || a.rows_lp > 0 || !scan_list_supported(P->nw, P->nwy, P->nbeams)) return;
     const long long n = (long long)sc->px * sc->py;
-    const bool large = P->nw >= 128;
-    if (n > 0 && (large ? n < 64 : sc->py < 8 || n < 2048)) {
-        a.list = 1;
-        return;
+    if (P->prec != PRISM_PRECISION_FP32 || a.rows_lp > 0 || n == 0 || !scan_list_supported(P->nw, P->nwy, P->nbeams)) return;
+    const int bx = (sc->px + 3) / 4, by = (sc->py + 7) / 8;
+    const long long blocks = (long long)bx * by, seen = std::min<long long>(blocks, 16);
+    const double np = (double)P->nw * P->nwy, B = P->nbeams;
+    long long apart = 0;
+    double area = 0;  // pixels of the union tiles
+    for (long long s = 0; s < seen; ++s) {
+        const long long k = s * blocks / seen;
+        const int r0 = (int)(k / bx) * 8, c0 = (int)(k % bx) * 4;
+        const int r1 = std::min(r0 + 8, sc->py), c1 = std::min(c0 + 4, sc->px);
+        double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
+        for (int r = r0; r < r1; ++r)
+            for (int c = c0; c < c1; ++c) {
+                const size_t q = (size_t)r * sc->px + c;
+                x0 = std::min(x0, sc->x0[q]);
+                x1 = std::max(x1, sc->x0[q]);
+                y0 = std::min(y0, sc->y0[q]);
+                y1 = std::max(y1, sc->y0[q]);
+            }
+        const double tile = ((x1 - x0) / a.px_s + P->nw) * ((y1 - y0) / a.py_s + P->nwy), own = (double)(r1 - r0) * (c1 - c0) * np;
+        apart += tile > own;
+        area += tile > own ? 8.0 * own : tile;  // (probe by probe one warp of eight works)
     }
-    long long apart = 0, blocks = 0;
-    for (int by = 0; by < sc->py; by += 8)
-        for (int bx = 0; bx < sc->px; bx += 4) {
-            const int ny = std::min(8, sc->py - by), nx = std::min(4, sc->px - bx);
-            double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
-            for (int j = by; j < by + ny; ++j)
-                for (int i = bx; i < bx + nx; ++i) {
-                    const size_t q = (size_t)j * sc->px + i;
-                    x0 = std::min(x0, sc->x0[q]);
-                    x1 = std::max(x1, sc->x0[q]);
-                    y0 = std::min(y0, sc->y0[q]);
-                    y1 = std::max(y1, sc->y0[q]);
-                }
-            ++blocks;
-            apart += ((x1 - x0) / a.px_s + P->nw) * ((y1 - y0) / a.py_s + P->nwy) > (double)nx * ny * P->nw * P->nwy;
-        }
-    a.list = blocks > 0 && 2 * apart >= blocks;
+    if (2 * apart >= seen) {
+        a.list = 1;
+    } else if (P->nw >= 128) {
+        a.list = n < 64 && n * B < 8000;
+    } else {
+        const double rounds = std::max(1.0, blocks / 304.0), parts = blocks < 304 ? (double)std::min(16LL, 304 / blocks) : 1.0;
+        const double reach = 8.0 * B * std::min(area / seen * blocks, (double)P->nxs * P->nys);  // bytes of S
+        const double list = 19.0 + n * (2.5e-3 + np * (7.7e-6 + (np < 4096 ? 4.3e-7 : reach < 80e6 ? 6.5e-7 : 1e-6) * B));
+        const double gemm = rounds * (19.0 + 1e-3 * B * area / seen / parts + 1.33e-3 * np * std::min(32.0, (double)n / blocks));
+        a.list = list < 0.95 * gemm;
+    }
 }
 
 static int scan_prepare(prism_plan *P, const prism_probe *probe, const prism_scan *sc, const prism_detector *det,

@@ -229,3 +229,23 @@ def test_list_sums_over_beams():
     assert i.n_beams == len(m) == 213
     assert np.sqrt(num / den) <= 0.425 * 2.0 ** -24 * np.sqrt(213 / 2 + 20)
     sim.close()
+
+
+@pytest.mark.parametrize("n,cell,f,px,py,step,path", [
+    (512, 32.0, 4, 16, 16, 0.1, P.PRISM_SCAN_LIST),      # 213 beams, 64-pixel windows: few probes
+    (512, 32.0, 4, 40, 40, 0.1, P.PRISM_SCAN_BLOCKS),    # blocks that share tiles
+    (512, 32.0, 4, 4, 200, 0.25, P.PRISM_SCAN_BLOCKS),
+    (512, 32.0, 4, 40, 40, 11.0, P.PRISM_SCAN_LIST),     # windows further apart than that
+    (128, 12.8, 2, 45, 45, 0.1, P.PRISM_SCAN_BLOCKS),    # 137 beams, 32-pixel windows
+    (256, 16.0, 4, 30, 30, 0.3, P.PRISM_SCAN_LIST),      # 49 beams
+    (128, 8.0, 4, 101, 97, 0.1, P.PRISM_SCAN_BLOCKS),    # 13 beams, 16-pixel windows
+    (1024, 50.0, 4, 10, 1, 0.3, P.PRISM_SCAN_LIST),      # 505 beams, 128-pixel windows
+    (1024, 50.0, 4, 20, 1, 0.3, P.PRISM_SCAN_BLOCKS),
+])
+def test_jittered_rasters_take_the_faster_path(n, cell, f, px, py, step, path):
+    sim = plan(n, cell, f, 11)
+    pos = jittered(px, py, step, 11)
+    out = scan(sim, pos, px, py, path)
+    some = np.array([0, px * py // 2, px * py - 1])
+    close(out[some], exact(sim, cell, f, 0, pos[0][some], pos[1][some]), sim.info.n_beams)
+    sim.close()
