@@ -999,8 +999,13 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
     const size_t row = (size_t)P->nwy * planes * cols * sizeof(float2);
     const size_t blocks = ((size_t)sc->px + 3) / 4 * (((size_t)sc->py + 3) / 4);
     size_t most = std::min<size_t>(blocks, 304) * 64 * P->nw * P->nwy * sizeof(float2);
-    // (under a caller's tight budget no more than the blocks would take of this very scan)
+    // Where no HBM budget is given, at least 128 MB: a tall raster of few columns has few blocks, and the rows
+    // that their scratch held went launch by launch (value + remainder storage, 4 x 99 probes of 49 beams and
+    // 32-pixel windows: 56 us on the tensor cores, 1031 us one row at a time; 3 x 75 of 213 beams and
+    // 64-pixel windows: 132, 334).  Under a batch's tight budget no more than the blocks would take of
+    // this very scan.
     if (P->scratch_budget) most = std::min(most, block_scratch(P, sc->px, sc->py));
+    else if (!P->budget) most = std::max<size_t>(most, (size_t)128 << 20);
     const size_t unpacked = split ? (size_t)P->nbeams * rows * cols * sizeof(float2) : 0;
     if (unpacked + row > most) return;
     const size_t limit = std::min<size_t>(most - unpacked, (size_t)384 << 20);
@@ -1009,6 +1014,9 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
     // in equal shares, to whole groups of 4
     chunk = ((size_t)sc->py + (sc->py + chunk - 1) / chunk - 1) / ((sc->py + chunk - 1) / chunk);
     if (chunk % 4 && chunk < (size_t)sc->py && (chunk + 3) / 4 * 4 * row <= limit) chunk = (chunk + 3) / 4 * 4;
+    // (value + remainder: in more than two launches each of fewer than 1024 probes the tensor cores are faster, in
+    // up to two they never were by more than 2 %)
+    if (split && ((size_t)sc->py + chunk - 1) / chunk > 2 && chunk * sc->px < 1024) return;
     const int lp = scan_rows_lp(P->nw, P->nwy, P->rows_m, P->rows_maxn, a.n_fold16, sc->px, (int)chunk);
     if (lp <= 0) return;
     a.rows_lp = lp;

@@ -17,8 +17,8 @@ DET = P.make_detector(0.0, 2.0, 40)
 PROBE = P.make_probe(20.0, 12.0)
 
 
-def plan(n, cell, f, seed, f_y=0, alpha=20.0, precision=P.PRISM_PRECISION_FP32):
-    sim = PrismSimulation(P.make_grid(n, n, 1, cell, cell, 2.0, 300.0, f, 2, 0.5, alpha, f_y=f_y, precision=precision))
+def plan(n, cell, f, seed, f_y=0, alpha=20.0, precision=P.PRISM_PRECISION_FP32, budget=0):
+    sim = PrismSimulation(P.make_grid(n, n, 1, cell, cell, 2.0, 300.0, f, 2, 0.5, alpha, f_y=f_y, precision=precision), budget)
     i = sim.info
     g = torch.Generator(device="cuda").manual_seed(seed)
     sim.load_smatrix(torch.view_as_complex(torch.randn((i.n_beams, i.ny_s, i.nx_s, 2), generator=g, device="cuda")))
@@ -248,4 +248,29 @@ def test_jittered_rasters_take_the_faster_path(n, cell, f, px, py, step, path):
     out = scan(sim, pos, px, py, path)
     some = np.array([0, px * py // 2, px * py - 1])
     close(out[some], exact(sim, cell, f, 0, pos[0][some], pos[1][some]), sim.info.n_beams)
+    sim.close()
+
+
+@pytest.mark.parametrize("n,cell,f,px,py,step", [
+    (512, 32.0, 8, 4, 99, 0.6),     # 32-pixel windows: the blocks' scratch holds one row at a time
+    (512, 32.0, 4, 3, 75, 0.31),    # 64-pixel windows, 213 beams
+    (128, 12.8, 2, 6, 6, 0.1),      # partial blocks, all split
+])
+@pytest.mark.parametrize("budget,path", [(0, P.PRISM_SCAN_ROWS), (1 << 33, P.PRISM_SCAN_TENSOR)])
+def test_narrow_value_and_remainder_rasters(n, cell, f, px, py, step, budget, path):
+    # by rows in one or two launches where memory is free, else by tensor-core blocks in split mode: never in many
+    # launches of a few rows
+    # a raster by tensor-core blocks in split mode or by rows, against 64 bits: 22-bit values and coefficients, and
+    # remainder x remainder left out, are at most 2^-20 of each product
+    sim = plan(n, cell, f, 12, precision=P.PRISM_PRECISION_FP16X2, budget=budget)
+    x, y = np.meshgrid(step * np.arange(px) - 1.3, step * np.arange(py) - 0.7)
+    pos = (x.ravel(), y.ravel())
+    out = scan(sim, pos, px, py, path)
+    some = np.array([0, px - 1, px * py // 2, px * py - 1])
+    ref = exact(sim, cell, f, 0, pos[0][some], pos[1][some])
+    err = np.linalg.norm(out[some] - ref) / np.linalg.norm(ref)
+    assert err <= 2.0 * (2.0 ** -20 * sim.info.n_beams ** 0.5 + (sim.info.n_beams + 24) * 2.0 ** -24), err
+    before = sim.launches()
+    assert np.array_equal(scan(sim, pos, px, py, path), out)
+    assert sim.launches() - before <= (5 if path == P.PRISM_SCAN_ROWS else 1)
     sim.close()
