@@ -967,6 +967,9 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, ScanArgs &a) 
     if ((P->prec != PRISM_PRECISION_FP32 && !split) || sc->px < 3 || sc->py < 1) return;
     // (up to 24 FP32 probes are as fast probe by probe, or faster: 4 x 4 of 129 beams 66 us by rows, 36 so)
     if (!split && P->nw < 128 && (long long)sc->px * sc->py <= 24) return;
+    // (value + remainder, one or two rows of 16-pixel windows: three launches, 24 us, where one on the tensor cores
+    // takes 21, no longer than it takes to launch)
+    if (split && P->nw <= 16 && sc->py <= 2) return;
     double xmin = sc->x0[0], xmax = sc->x0[0], ymin = sc->y0[0], ymax = sc->y0[0];
     for (int r = 0; r < sc->py; ++r) {
         const double *x = sc->x0 + (size_t)r * sc->px, *y = sc->y0 + (size_t)r * sc->px;

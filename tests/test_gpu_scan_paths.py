@@ -274,3 +274,14 @@ def test_narrow_value_and_remainder_rasters(n, cell, f, px, py, step, budget, pa
     assert np.array_equal(scan(sim, pos, px, py, path), out)
     assert sim.launches() - before <= (5 if path == P.PRISM_SCAN_ROWS else 1)
     sim.close()
+
+
+@pytest.mark.parametrize("py", [1, 2, 3])
+def test_few_rows_of_small_value_and_remainder_windows(py):
+    sim = plan(128, 8.0, 4, 13, precision=P.PRISM_PRECISION_FP16X2)
+    x, y = np.meshgrid(0.2 * np.arange(47), 0.2 * np.arange(py))
+    pos = (x.ravel(), y.ravel())
+    out = scan(sim, pos, 47, py, P.PRISM_SCAN_TENSOR if py <= 2 else P.PRISM_SCAN_ROWS)
+    ref = exact(sim, 8.0, 4, 0, *pos)
+    assert np.linalg.norm(out - ref) / np.linalg.norm(ref) <= 2.0 * (2.0 ** -20 * 13 ** 0.5 + (13 + 24) * 2.0 ** -24)
+    sim.close()
