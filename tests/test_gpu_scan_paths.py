@@ -285,3 +285,29 @@ def test_few_rows_of_small_value_and_remainder_windows(py):
     ref = exact(sim, 8.0, 4, 0, *pos)
     assert np.linalg.norm(out - ref) / np.linalg.norm(ref) <= 2.0 * (2.0 ** -20 * 13 ** 0.5 + (13 + 24) * 2.0 ** -24)
     sim.close()
+
+
+@pytest.mark.parametrize("px,py", [(11, 9), (7, 16), (1, 130), (130, 1)])
+def test_positions_are_checked_everywhere(px, py):
+    # a NaN, an infinity or a position beyond 2^28 pixels anywhere among them is refused; the largest position
+    # allowed, and rows whose y are zeros of both signs, are not
+    sim = plan(128, 8.0, 4, 14)
+    x, y = np.meshgrid(0.2 * np.arange(px), 0.2 * np.arange(py))
+    pos = [x.ravel(), y.ravel()]
+    ref = sim.scan(PROBE, *pos, DET, px=px, py=py).cpu().numpy()
+    path = P.prism_plan_scan_path(sim.plan)
+    for axis in (0, 1):
+        for at in sorted({0, 1, 5, px * py // 2, px * py - 2, px * py - 1}):
+            for bad in (np.nan, -np.nan, np.inf, -np.inf, 2.0 ** 28 * 0.125 * (1 + 2.0 ** -50), -1e300):
+                p = [q.copy() for q in pos]
+                p[axis][at] = bad
+                with pytest.raises(P.PrismError) as e:
+                    sim.scan(PROBE, *p, DET, px=px, py=py)
+                assert e.value.status == P.PRISM_ERR_INVALID
+    p = [q.copy() for q in pos]
+    p[1][: px : 2] = -0.0
+    assert np.array_equal(sim.scan(PROBE, *p, DET, px=px, py=py).cpu().numpy(), ref)
+    assert P.prism_plan_scan_path(sim.plan) == path
+    p[0][:] = 2.0 ** 28 * 0.125
+    sim.scan(PROBE, *p, DET, px=px, py=py)
+    sim.close()
