@@ -447,8 +447,8 @@ struct prism_plan {
     void *S16 = nullptr;       // 16-bit mode: [ny_s * nx_s][kp]
     float *scale = nullptr;    // 16-bit mode: [kp / 2] per-beam power-of-two scales
     int kp = 0;
-    float2 *win = nullptr;     // scan window scratch (GEMM and tensor-core scans)
-    size_t win_cap = 0;
+    float2 *win = nullptr;     // scan scratch, of whichever way the scan takes: windows of the GEMM and tensor-core
+    size_t win_cap = 0;        // scans; sums over n of the raster-row scan, then its unpacked S-matrix
     int *win_cnt = nullptr;    // scans: completion counters of split groups, work-unit counters
     size_t cnt_cap = 0;
     CUtensorMap wave_map, wave_map4;  // the wave stack for the TMA-staged column pass (8 / 4 columns per box)
@@ -475,11 +475,7 @@ struct prism_plan {
     int *m_off = nullptr, *m_beam = nullptr;  // the beams by m (ScanArgs::m_off)
     double *m_qx = nullptr;
     int rows_m = 0, rows_maxn = 0;
-    float2 *rows_w = nullptr;  // sums over n of the raster-row scan
-    size_t rows_cap = 0;
     bool rows_attrs = false, list_attrs = false;  // the kernels' shared-memory limits have been set
-    float2 *rows_s = nullptr;  // what the windows reach of a value + remainder S-matrix, unpacked
-    size_t rows_s_cap = 0;
     // grown on demand
     double *pos = nullptr;
     size_t pos_cap = 0;
@@ -1307,12 +1303,12 @@ static int tc_shape(const prism_plan *P) {
 static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
     *grid = 0;
     if (a.rows_lp > 0) {
-        const size_t wb = (size_t)a.rows_chunk * P->nwy * (2 * a.rows_m + 1) * a.rows_cols * sizeof(float2);
-        int rc = grow(P->arena, (void **)&P->rows_w, &P->rows_cap, wb);
-        if (!rc && a.rows_unpack) rc = grow(P->arena, (void **)&P->rows_s, &P->rows_s_cap, scan_rows_unpack_bytes(a));
+        // (rows_cols is a multiple of 16: both parts start on 128 bytes)
+        const size_t sums = (size_t)a.rows_chunk * P->nwy * (2 * a.rows_m + 1) * a.rows_cols;
+        const int rc = grow(P->arena, (void **)&P->win, &P->win_cap, sums * sizeof(float2) + (a.rows_unpack ? scan_rows_unpack_bytes(a) : 0));
         if (!rc) {
-            a.rows_w = P->rows_w;
-            a.rows_src = a.rows_unpack ? P->rows_s : P->S;
+            a.rows_w = P->win;
+            a.rows_src = a.rows_unpack ? P->win + sums : P->S;
             *grid = 1;
             return PRISM_OK;
         }
@@ -2230,10 +2226,9 @@ extern "C" int prism_batch_create(const prism_cell *cells, int n_cells, size_t h
             ScanArgs &a = B->scans[i];
             if (a.rows_lp > 0) {
                 P->scratch_budget = true;
-                if (P->rows_w) P->arena.forget(P->rows_w, P->rows_cap);
-                if (P->rows_s) P->arena.forget(P->rows_s, P->rows_s_cap);
-                P->rows_w = P->rows_s = nullptr;
-                P->rows_cap = P->rows_s_cap = 0;
+                if (P->win) P->arena.forget(P->win, P->win_cap);
+                P->win = nullptr;
+                P->win_cap = 0;
                 if ((rc = scan_prepare(P, &cells[i].probe, &cells[i].scan, &cells[i].det, a, false)) || (rc = scan_setup(P, a, &B->scan_grid[i])))
                     return fail(rc, "cell " + std::to_string(i) + ": " + g_err), bail(rc);
                 a.out = cells[i].out_dev;

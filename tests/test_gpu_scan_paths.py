@@ -311,3 +311,28 @@ def test_positions_are_checked_everywhere(px, py):
     p[0][:] = 2.0 ** 28 * 0.125
     sim.scan(PROBE, *p, DET, px=px, py=py)
     sim.close()
+
+
+@pytest.mark.parametrize("precision", [P.PRISM_PRECISION_FP32, P.PRISM_PRECISION_FP16X2])
+def test_a_plan_holds_the_scratch_of_one_path(precision):
+    # a plan that scans by rows and by blocks in turn keeps one scratch, as large as the larger needs
+    def held(sim):
+        return P.prism_plan_info(sim.plan).device_bytes
+
+    x, y = np.meshgrid(0.2 * np.arange(60), 0.15 * np.arange(80))
+    rows, off = (x.ravel(), y.ravel()), jittered(60, 80, 0.2, 15)
+    other = P.PRISM_SCAN_BLOCKS if precision == P.PRISM_PRECISION_FP32 else P.PRISM_SCAN_TENSOR
+    alone = []
+    for pos, path in ((rows, P.PRISM_SCAN_ROWS), (off, other)):
+        sim = plan(256, 16.0, 2, 15, precision=precision)
+        base = held(sim)
+        out = scan(sim, pos, 60, 80, path)
+        alone.append((held(sim) - base, out))
+        sim.close()
+    sim = plan(256, 16.0, 2, 15, precision=precision)
+    for _ in range(2):
+        assert np.array_equal(scan(sim, rows, 60, 80, P.PRISM_SCAN_ROWS), alone[0][1])
+        assert np.array_equal(scan(sim, off, 60, 80, other), alone[1][1])
+    assert min(a for a, _ in alone) > 1 << 20
+    assert held(sim) - base <= max(a for a, _ in alone) + (1 << 16)  # (counters)
+    sim.close()
