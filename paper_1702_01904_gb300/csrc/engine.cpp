@@ -1300,7 +1300,7 @@ static int tc_shape(const prism_plan *P) {
     return P->tc_shape > 0 && P->tc_shape < scan_tc_shapes(tc_mode(P->prec)) ? P->tc_shape : 0;
 }
 
-static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
+static int scan_setup(prism_plan *P, const prism_scan *sc, ScanArgs &a, int *grid) {
     *grid = 0;
     if (a.rows_lp > 0) {
         // (rows_cols is a multiple of 16: both parts start on 128 bytes)
@@ -1312,8 +1312,12 @@ static int scan_setup(prism_plan *P, ScanArgs &a, int *grid) {
             *grid = 1;
             return PRISM_OK;
         }
-        cudaGetLastError();  // no memory for the rows: in blocks, whose scratch is smaller for long rasters
-        a.rows_lp = 0;
+        // no memory for the rows: as positions of any raster, probe by probe or in blocks, whose scratch is smaller
+        // for long rasters
+        cudaGetLastError();
+        a.rows_lp = a.rows_unpack = 0;
+        position_list(P, sc, a);
+        a.attrs_set = P->list_attrs;
     }
     if (a.list) {
         *grid = 1;
@@ -1365,9 +1369,9 @@ static int scan_go(prism_plan *P, const ScanArgs &a, int grid) {
     return plan_launch(P, PRISM_K_SCAN, [&] { return launch_scan_tc(P->nw, tc_mode(P->prec), tc_shape(P), grid, a, P->stream); });
 }
 
-static int scan_launch(prism_plan *P, ScanArgs &a) {
+static int scan_launch(prism_plan *P, const prism_scan *sc, ScanArgs &a) {
     int grid = 0;
-    int rc = scan_setup(P, a, &grid);
+    int rc = scan_setup(P, sc, a, &grid);
     if (rc) return rc;
     return scan_go(P, a, grid);
 }
@@ -1381,7 +1385,7 @@ extern "C" int prism_scan_run(prism_plan *P, const prism_probe *probe, const pri
     if (a.n_probes == 0) return PRISM_OK;
     if ((rc = check_dev_ptr(out_dev, 4, "out_dev"))) return rc;
     a.out = out_dev;
-    return scan_launch(P, a);
+    return scan_launch(P, sc, a);
 }
 
 extern "C" int prism_scan_run_host(prism_plan *P, const prism_probe *probe, const prism_scan *sc,
@@ -1395,7 +1399,7 @@ extern "C" int prism_scan_run_host(prism_plan *P, const prism_probe *probe, cons
     const size_t bytes = (size_t)a.n_probes * det->nbins * sizeof(float);
     if ((rc = grow(P->arena, (void **)&P->out_stage, &P->out_cap, bytes))) return rc;
     a.out = P->out_stage;
-    rc = scan_launch(P, a);
+    rc = scan_launch(P, sc, a);
     if (rc) return rc;
     CUDA_TRY(cudaMemcpyAsync(out_host, P->out_stage, bytes, cudaMemcpyDeviceToHost, P->stream));
     return PRISM_OK;
@@ -1410,7 +1414,7 @@ extern "C" int prism_scan_run_cbed(prism_plan *P, const prism_probe *probe, cons
     if ((rc = check_dev_ptr(out_dev, 4, "out_dev"))) return rc;
     a.out = nullptr;
     a.cbed = out_dev;
-    return scan_launch(P, a);
+    return scan_launch(P, sc, a);
 }
 
 extern "C" int prism_scan_run_accumulate(prism_plan *P, const prism_probe *probe, const prism_scan *sc,
@@ -1425,7 +1429,7 @@ extern "C" int prism_scan_run_accumulate(prism_plan *P, const prism_probe *probe
     a.out = out_dev;
     a.accumulate = 1;
     a.acc_w = weight;
-    return scan_launch(P, a);
+    return scan_launch(P, sc, a);
 }
 
 // ------------------------------------------------------------------ multislice baseline
@@ -2034,7 +2038,7 @@ extern "C" int prism_tune_shape_fft_variant(int kind, int shape) {
 // 16-bit plans: time the caller's scan with each ring shape of the tensor-core scan (a warm-up and
 // two timed launches each) and keep the fastest; every shape gives bitwise the same stack, which
 // is left in a.out
-static int autotune_scan_tc(prism_plan *P, ScanArgs &a) {
+static int autotune_scan_tc(prism_plan *P, const prism_scan *sc, ScanArgs &a) {
     for (int v = 0; v < PRISM_TUNE_MAX_SHAPES; ++v) P->tc_ms[v] = -1.0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CUDA_TRY(cudaEventCreate(&e0));
@@ -2045,7 +2049,7 @@ static int autotune_scan_tc(prism_plan *P, ScanArgs &a) {
         P->tc_shape = v;
         int grid = 0;
         if (scan_tc_grid(P->nw, P->kp, tc_mode(P->prec), v, a.scan_px, a.scan_py) <= 0) continue;  // does not fit
-        if ((rc = scan_setup(P, a, &grid))) break;
+        if ((rc = scan_setup(P, sc, a, &grid))) break;
         if ((rc = scan_go(P, a, grid))) break;
         cudaError_t e = cudaEventRecord(e0, P->stream);
         for (int r = 0; r < 2 && e == cudaSuccess && !rc; ++r) rc = scan_go(P, a, grid);
@@ -2069,7 +2073,7 @@ static int autotune_scan_tc(prism_plan *P, ScanArgs &a) {
     P->tc_shape = best;
     P->tc_tuned = !rc;
     if (rc) return rc;
-    return scan_launch(P, a);
+    return scan_launch(P, sc, a);
 }
 
 // The scan's contraction tile shape (Calculation Time section: the scan term P B N^2 / (4 f^4) is
@@ -2085,26 +2089,26 @@ extern "C" int prism_plan_autotune_scan(prism_plan *P, const prism_probe *probe,
     if (a.n_probes == 0) return PRISM_OK;
     if ((rc = check_dev_ptr(out_dev, 4, "out_dev"))) return rc;
     a.out = out_dev;
-    if (P->prec != PRISM_PRECISION_FP32) return autotune_scan_tc(P, a);
+    if (P->prec != PRISM_PRECISION_FP32) return autotune_scan_tc(P, sc, a);
     for (int v = 0; v < PRISM_TUNE_MAX_SHAPES; ++v) P->scan_ms[v] = -1.0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
     // a scan by raster rows or probe by probe has no contraction blocks: timed once, the same for every
-    // shape, and the plan's shape stays
-    const bool rows = a.rows_lp > 0 || a.list;
+    // shape, and the plan's shape stays (which way it goes is known once its scratch is allocated)
     const int kept = P->scan_shape;
-    int best = rows ? kept : 0;
+    int best = 0;
     double best_ms = -1.0;
     for (int v = 0; v < scan_gemm_shapes() && v < PRISM_TUNE_MAX_SHAPES && !rc; ++v) {
         if (!scan_gemm_shape_valid(P->nw, P->nwy, v)) continue;
-        if (rows && best_ms >= 0) {
+        if (best_ms >= 0 && (a.rows_lp > 0 || a.list)) {
             P->scan_ms[v] = best_ms;
             continue;
         }
-        if (!rows) P->scan_shape = v;
+        P->scan_shape = v;
         int grid = 0;
-        if ((rc = scan_setup(P, a, &grid))) break;
+        if ((rc = scan_setup(P, sc, a, &grid))) break;
+        const bool rows = a.rows_lp > 0 || a.list;
         if (grid <= 0) continue;  // this shape's coefficient block does not fit shared memory
         if ((rc = scan_go(P, a, grid))) break;
         cudaError_t e = cudaEventRecord(e0, P->stream);
@@ -2129,7 +2133,7 @@ extern "C" int prism_plan_autotune_scan(prism_plan *P, const prism_probe *probe,
     P->scan_shape = best;
     P->scan_tuned = !rc;
     if (rc) return rc;
-    return scan_launch(P, a);  // the detector stack of the chosen shape (bitwise that of every shape)
+    return scan_launch(P, sc, a);  // the detector stack of the chosen shape (bitwise that of every shape)
 }
 
 // ------------------------------------------------------------------ batches of cells (one CUDA graph)
@@ -2209,7 +2213,7 @@ extern "C" int prism_batch_create(const prism_cell *cells, int n_cells, size_t h
         if ((rc = scan_prepare(P, &c.probe, &c.scan, &c.det, a, false))) return fail(rc, "cell " + std::to_string(i) + ": " + g_err), bail(rc);
         a.out = c.out_dev;
         int grid = 0;
-        if (a.n_probes > 0 && (rc = scan_setup(P, a, &grid))) return bail(rc);
+        if (a.n_probes > 0 && (rc = scan_setup(P, &c.scan, a, &grid))) return bail(rc);
         B->scans.push_back(a);
         B->scan_grid.push_back(grid);
         B->V.push_back(c.V_dev);
@@ -2229,7 +2233,7 @@ extern "C" int prism_batch_create(const prism_cell *cells, int n_cells, size_t h
                 if (P->win) P->arena.forget(P->win, P->win_cap);
                 P->win = nullptr;
                 P->win_cap = 0;
-                if ((rc = scan_prepare(P, &cells[i].probe, &cells[i].scan, &cells[i].det, a, false)) || (rc = scan_setup(P, a, &B->scan_grid[i])))
+                if ((rc = scan_prepare(P, &cells[i].probe, &cells[i].scan, &cells[i].det, a, false)) || (rc = scan_setup(P, &cells[i].scan, a, &B->scan_grid[i])))
                     return fail(rc, "cell " + std::to_string(i) + ": " + g_err), bail(rc);
                 a.out = cells[i].out_dev;
             }

@@ -1,6 +1,7 @@
 """Every kernel that a scan can take, with the path asserted: the block scan's contraction shapes, split blocks,
 work-unit counters, scratch and shared-memory limits on positions that go by blocks (rasters of many probes
 whose rows do not share a y, tall rasters of two columns)."""
+import ctypes
 import threading
 
 import numpy as np
@@ -336,3 +337,65 @@ def test_a_plan_holds_the_scratch_of_one_path(precision):
     assert min(a for a, _ in alone) > 1 << 20
     assert held(sim) - base <= max(a for a, _ in alone) + (1 << 16)  # (counters)
     sim.close()
+
+
+class SmallPool:
+    """Device memory for the library's stream-ordered allocations up to `mb` megabytes (a multiple of 32, the
+    grain of a pool), through a memory pool of that size in the place of the device's own."""
+
+    class Props(ctypes.Structure):
+        class Location(ctypes.Structure):
+            _fields_ = [("type", ctypes.c_int), ("id", ctypes.c_int)]
+
+        _fields_ = [("alloc", ctypes.c_int), ("handles", ctypes.c_int), ("location", Location), ("win32", ctypes.c_void_p),
+                    ("max_size", ctypes.c_size_t), ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
+
+    def __init__(self, mb):
+        self.cu = ctypes.CDLL("libcuda.so.1")
+        self.mb = mb
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        dev = torch.cuda.current_device()
+        self.own, self.pool = ctypes.c_void_p(), ctypes.c_void_p()
+        assert self.cu.cuDeviceGetDefaultMemPool(ctypes.byref(self.own), dev) == 0
+        p = self.Props(1, 0, self.Props.Location(1, dev), None, self.mb << 20, 0)  # pinned device memory
+        assert self.cu.cuMemPoolCreate(ctypes.byref(self.pool), ctypes.byref(p)) == 0
+        assert self.cu.cuDeviceSetMemPool(dev, self.pool) == 0
+        return self
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        assert self.cu.cuDeviceSetMemPool(torch.cuda.current_device(), self.own) == 0
+        assert self.cu.cuMemPoolDestroy(self.pool) == 0
+
+    def most_used(self):
+        v = ctypes.c_ulonglong()
+        assert self.cu.cuMemPoolGetAttribute(self.pool, 8, ctypes.byref(v)) == 0  # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+        return v.value
+
+
+@pytest.mark.parametrize("f,px,py,step,slack,path", [(4, 9, 125, 2.0, 4, P.PRISM_SCAN_LIST), (2, 4, 110, 0.5, 32, P.PRISM_SCAN_BLOCKS)])
+def test_rows_without_memory_take_another_path(f, px, py, step, slack, path):
+    # the rows' scratch does not fit beside the plan: the scan goes as positions off their rows would, and the
+    # autotuner times what then runs
+    x, y = np.meshgrid(step * np.arange(px), 0.14 * np.arange(py))
+    pos = (x.ravel(), y.ravel())
+    sim = plan(256, 16.0, f, 16)
+    need = sim.info.device_bytes
+    full = scan(sim, pos, px, py, P.PRISM_SCAN_ROWS)
+    rows = P.prism_plan_info(sim.plan).device_bytes - need
+    sim.close()
+    mb = (need + (slack << 20) + (1 << 25) - 1) // (1 << 25) * 32
+    assert need + rows > mb << 20
+    with SmallPool(mb):
+        sim = plan(256, 16.0, f, 16)
+        out = scan(sim, pos, px, py, path)
+        assert np.array_equal(scan(sim, pos, px, py, path), out)
+        tuned = sim.autotune_scan(PROBE, *pos, DET, px=px, py=py).cpu().numpy()
+        assert P.prism_plan_scan_path(sim.plan) == path and np.array_equal(tuned, out)
+        ms = set(sim.tune_result()["scan"]["ms"].values())
+        assert len(ms) == 1 if path == P.PRISM_SCAN_LIST else len(ms) > 1
+        beams = sim.info.n_beams
+        sim.close()
+    close(out, full.astype(np.float64), beams)
