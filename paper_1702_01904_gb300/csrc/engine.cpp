@@ -1300,16 +1300,39 @@ static int tc_shape(const prism_plan *P) {
     return P->tc_shape > 0 && P->tc_shape < scan_tc_shapes(tc_mode(P->prec)) ? P->tc_shape : 0;
 }
 
-static int scan_setup(prism_plan *P, const prism_scan *sc, ScanArgs &a, int *grid) {
-    *grid = 0;
+// The grid and the bytes of scratch (and of counters) of the path a scan takes; grid 0: kernels that need none
+static int scan_scratch(const prism_plan *P, const ScanArgs &a, int *grid, size_t *win, size_t *cnt) {
+    *grid = 1;
+    *win = *cnt = 0;
     if (a.rows_lp > 0) {
-        // (rows_cols is a multiple of 16: both parts start on 128 bytes)
-        const size_t sums = (size_t)a.rows_chunk * P->nwy * (2 * a.rows_m + 1) * a.rows_cols;
-        const int rc = grow(P->arena, (void **)&P->win, &P->win_cap, sums * sizeof(float2) + (a.rows_unpack ? scan_rows_unpack_bytes(a) : 0));
+        // (rows_cols is a multiple of 16: the unpacked values start on 128 bytes)
+        *win = (size_t)a.rows_chunk * P->nwy * (2 * a.rows_m + 1) * a.rows_cols * sizeof(float2) + (a.rows_unpack ? scan_rows_unpack_bytes(a) : 0);
+        return PRISM_OK;
+    }
+    if (a.list) return PRISM_OK;
+    if (P->prec == PRISM_PRECISION_FP32) {
+        const int sh = gemm_shape(P);
+        *grid = std::max(0, scan_gemm_grid(P->nw, P->nwy, sh, P->nbeams, a.scan_px, a.scan_py));
+        if (*grid == 0) return PRISM_OK;
+        *win = scan_gemm_win_bytes(P->nw, P->nwy, sh, *grid, a.scan_px, a.scan_py);
+        if (!*win) return fail(PRISM_ERR_CUDA, "FP32 scan: no window scratch size for contraction shape " + std::to_string(sh));
+    } else {
+        *grid = scan_tc_grid(P->nw, P->kp, tc_mode(P->prec), tc_shape(P), a.scan_px, a.scan_py);
+        if (*grid <= 0) return fail(PRISM_ERR_CUDA, "tensor-core scan: no resident launch configuration");
+        *win = scan_tc_win_bytes(P->nw, *grid, a.scan_px, a.scan_py);
+    }
+    *cnt = scan_gemm_cnt_bytes(*grid);
+    return PRISM_OK;
+}
+
+static int scan_setup(prism_plan *P, const prism_scan *sc, ScanArgs &a, int *grid) {
+    size_t win = 0, cnt = 0;
+    int rc = scan_scratch(P, a, grid, &win, &cnt);
+    if (!rc && win) rc = grow(P->arena, (void **)&P->win, &P->win_cap, win);
+    if (a.rows_lp > 0) {
         if (!rc) {
             a.rows_w = P->win;
-            a.rows_src = a.rows_unpack ? P->win + sums : P->S;
-            *grid = 1;
+            a.rows_src = a.rows_unpack ? P->win + (win - scan_rows_unpack_bytes(a)) / sizeof(float2) : P->S;
             return PRISM_OK;
         }
         // no memory for the rows: as positions of any raster, probe by probe or in blocks, whose scratch is smaller
@@ -1318,29 +1341,9 @@ static int scan_setup(prism_plan *P, const prism_scan *sc, ScanArgs &a, int *gri
         a.rows_lp = a.rows_unpack = 0;
         position_list(P, sc, a);
         a.attrs_set = P->list_attrs;
+        return scan_setup(P, sc, a, grid);
     }
-    if (a.list) {
-        *grid = 1;
-        return PRISM_OK;
-    }
-    if (P->prec == PRISM_PRECISION_FP32) {
-        const int sh = gemm_shape(P);
-        *grid = scan_gemm_grid(P->nw, P->nwy, sh, P->nbeams, a.scan_px, a.scan_py);
-        if (*grid <= 0) {
-            *grid = 0;
-            return PRISM_OK;
-        }
-        const size_t wb = scan_gemm_win_bytes(P->nw, P->nwy, sh, *grid, a.scan_px, a.scan_py);
-        if (!wb) return fail(PRISM_ERR_CUDA, "FP32 scan: no window scratch size for contraction shape " + std::to_string(sh));
-        int rc = grow(P->arena, (void **)&P->win, &P->win_cap, wb);
-        if (rc) return rc;
-        return split_counters(P, a, *grid);
-    }
-    *grid = scan_tc_grid(P->nw, P->kp, tc_mode(P->prec), tc_shape(P), a.scan_px, a.scan_py);
-    if (*grid <= 0) return fail(PRISM_ERR_CUDA, "tensor-core scan: no resident launch configuration");
-    int rc = grow(P->arena, (void **)&P->win, &P->win_cap, scan_tc_win_bytes(P->nw, *grid, a.scan_px, a.scan_py));
-    if (rc) return rc;
-    return split_counters(P, a, *grid);
+    return rc || !cnt ? rc : split_counters(P, a, *grid);
 }
 
 static int scan_go(prism_plan *P, const ScanArgs &a, int grid) {
@@ -2199,7 +2202,6 @@ extern "C" int prism_batch_create(const prism_cell *cells, int n_cells, size_t h
     if ((e = cudaStreamCreateWithFlags(&B->origin, cudaStreamNonBlocking)) != cudaSuccess) return cuda_bail(e, "stream");
     // plans on the origin stream first (their allocations and uploads), branches assigned after
     std::vector<double> cost(n_cells);
-    size_t bytes = 0;
     for (int i = 0; i < n_cells; ++i) {
         const prism_cell &c = cells[i];
         prism_plan *P = nullptr;
@@ -2212,36 +2214,57 @@ extern "C" int prism_batch_create(const prism_cell *cells, int n_cells, size_t h
         ScanArgs a;
         if ((rc = scan_prepare(P, &c.probe, &c.scan, &c.det, a, false))) return fail(rc, "cell " + std::to_string(i) + ": " + g_err), bail(rc);
         a.out = c.out_dev;
-        int grid = 0;
-        if (a.n_probes > 0 && (rc = scan_setup(P, &c.scan, a, &grid))) return bail(rc);
         B->scans.push_back(a);
-        B->scan_grid.push_back(grid);
+        B->scan_grid.push_back(0);
         B->V.push_back(c.V_dev);
-        bytes += P->arena.bytes;
         const double px = (double)c.grid.nx * c.grid.ny;
         cost[i] = (double)P->nbeams * c.grid.n_slices * px * 32.0 +
                   (double)a.n_probes * P->nbeams * P->nw * P->nwy * (P->prec == PRISM_PRECISION_FP32 ? 8.0 : 1.0);
     }
-    // over the budget with the scratch of the raster-row scans: again with no more than the block scans take
-    if (hbm_budget_bytes && bytes > hbm_budget_bytes) {
-        bytes = 0;
+    // the scans' scratch, once every plan has its memory: what it takes is known before any of it is allocated.
+    // Over the budget, or without the memory, the rasters that go by rows are prepared again with no more
+    // scratch than the block scans take.
+    const auto needed = [&](size_t *bytes) {
+        *bytes = 0;
+        for (int i = 0; i < n_cells; ++i) {
+            size_t win = 0, cnt = 0;
+            int rc = PRISM_OK;
+            if (B->scans[i].n_probes > 0 && (rc = scan_scratch(B->plans[i], B->scans[i], &B->scan_grid[i], &win, &cnt))) return rc;
+            *bytes += B->plans[i]->arena.bytes + win + cnt;
+        }
+        return (int)PRISM_OK;
+    };
+    const auto least = [&] {
         for (int i = 0; i < n_cells; ++i) {
             prism_plan *P = B->plans[i];
-            ScanArgs &a = B->scans[i];
-            if (a.rows_lp > 0) {
-                P->scratch_budget = true;
-                if (P->win) P->arena.forget(P->win, P->win_cap);
-                P->win = nullptr;
-                P->win_cap = 0;
-                if ((rc = scan_prepare(P, &cells[i].probe, &cells[i].scan, &cells[i].det, a, false)) || (rc = scan_setup(P, &cells[i].scan, a, &B->scan_grid[i])))
-                    return fail(rc, "cell " + std::to_string(i) + ": " + g_err), bail(rc);
-                a.out = cells[i].out_dev;
-            }
-            bytes += P->arena.bytes;
+            if (P->win) P->arena.forget(P->win, P->win_cap);
+            P->win = nullptr;
+            P->win_cap = 0;
+            P->scratch_budget = true;
+            if (B->scans[i].n_probes == 0) continue;
+            const int rc = scan_prepare(P, &cells[i].probe, &cells[i].scan, &cells[i].det, B->scans[i], false);
+            if (rc) return fail(rc, "cell " + std::to_string(i) + ": " + g_err);
+            B->scans[i].out = cells[i].out_dev;
         }
-    }
+        return (int)PRISM_OK;
+    };
+    size_t bytes = 0;
+    if ((rc = needed(&bytes))) return bail(rc);
+    if (hbm_budget_bytes && bytes > hbm_budget_bytes && ((rc = least()) || (rc = needed(&bytes)))) return bail(rc);
     if (hbm_budget_bytes && bytes > hbm_budget_bytes)
         return fail(PRISM_ERR_BUDGET, "batch needs " + std::to_string(bytes) + " bytes, budget " + std::to_string(hbm_budget_bytes)), bail(PRISM_ERR_BUDGET);
+    const auto setup = [&] {
+        for (int i = 0; i < n_cells; ++i) {
+            int rc = PRISM_OK;
+            if (B->scans[i].n_probes > 0 && (rc = scan_setup(B->plans[i], &cells[i].scan, B->scans[i], &B->scan_grid[i])))
+                return fail(rc, "cell " + std::to_string(i) + ": " + g_err);
+        }
+        return (int)PRISM_OK;
+    };
+    if ((rc = setup())) {
+        cudaGetLastError();
+        if ((rc = least()) || (rc = setup())) return bail(rc);
+    }
     if ((e = cudaStreamSynchronize(B->origin)) != cudaSuccess) return cuda_bail(e, "batch setup");
     // longest estimated work first onto the least-loaded branch
     std::vector<int> order(n_cells);

@@ -2,6 +2,7 @@
 work-unit counters, scratch and shared-memory limits on positions that go by blocks (rasters of many probes
 whose rows do not share a y, tall rasters of two columns)."""
 import ctypes
+import re
 import threading
 
 import numpy as np
@@ -10,7 +11,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from paper_1702_01904_gb300 import prism as P  # noqa: E402
-from paper_1702_01904_gb300.runtime import PrismSimulation  # noqa: E402
+from paper_1702_01904_gb300.runtime import Batch, PrismSimulation  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -399,3 +400,52 @@ def test_rows_without_memory_take_another_path(f, px, py, step, slack, path):
         beams = sim.info.n_beams
         sim.close()
     close(out, full.astype(np.float64), beams)
+
+
+def rows_cell(seed, precision=P.PRISM_PRECISION_FP32):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x, y = np.meshgrid(0.5 * np.arange(4), 0.14 * np.arange(110))
+    return dict(grid=P.make_grid(256, 256, 1, 16.0, 16.0, 2.0, 300.0, 2, 2, 0.5, 20.0, precision=precision),
+                V=50.0 * torch.rand((1, 256, 256), generator=g, device="cuda"), probe=PROBE, x0=x.ravel(), y0=y.ravel(), px=4, py=110, det=DET)
+
+
+def run_batch(cells, budget=0):
+    b = Batch(cells, hbm_budget_bytes=budget, n_branches=1)
+    b.run()
+    b.sync()
+    out, held = [o.cpu().numpy() for o in b.outs], b.info.device_bytes
+    b.close()
+    return out, held
+
+
+def least_bytes(cells):
+    with pytest.raises(P.PrismError) as e:
+        Batch(cells, hbm_budget_bytes=1)
+    return int(re.search(r"batch needs (\d+) bytes", str(e.value)).group(1))
+
+
+def test_a_batch_stays_within_its_budget_throughout():
+    # the rows' scratch (some 120 MB a cell) is not allocated before the budget is looked at
+    cells = [rows_cell(s) for s in (17, 18)]
+    free, held = run_batch(cells)
+    least = least_bytes(cells)
+    assert held > least + (64 << 20)
+    with SmallPool(4096) as pool:
+        tight, used = run_batch(cells, least)
+        assert used == least
+        assert pool.most_used() <= least + (4 << 20)  # (allocations round up)
+    for a, b in zip(tight, free):
+        close(a, b.astype(np.float64), 213)
+
+
+def test_rows_leave_later_cells_their_memory():
+    # without a budget: the first cell's rows would leave no memory for the second cell's plan
+    cells = [rows_cell(s) for s in (19, 20)]
+    free, held = run_batch(cells)
+    mb = (least_bytes(cells) + (40 << 20)) // (1 << 25) * 32
+    assert held > mb << 20
+    with SmallPool(mb):
+        out, used = run_batch(cells)
+    assert used <= mb << 20
+    for a, b in zip(out, free):
+        close(a, b.astype(np.float64), 213)
