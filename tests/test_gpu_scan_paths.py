@@ -449,3 +449,34 @@ def test_rows_leave_later_cells_their_memory():
     assert used <= mb << 20
     for a, b in zip(out, free):
         close(a, b.astype(np.float64), 213)
+
+
+@pytest.mark.parametrize("n,cell,f,f_y,alpha,M,px,py,step", [
+    (256, 16.0, 4, 2, 4.0, 0, 40, 9, 0.2),       # m = 0 alone, three beams along y; 32 x 64 windows
+    (256, 16.0, 8, 4, 9.0, 0, 33, 5, 0.3),       # 16 x 32
+    (256, 16.0, 4, 0, 5.0, 1, 41, 6, 0.2),       # one pair of m
+    (256, 14.4, 2, 0, 25.0, 9, 12, 7, 0.3),      # 64 x 64, pairs of m in two chunks, three of them empty
+    (256, 14.4, 2, 0, 36.0, 13, 9, 5, 0.2),      # in two chunks of 7
+    (256, 16.0, 1, 0, 14.0, 11, 5, 6, 0.3),      # 128 x 128, two chunks
+])
+def test_rows_of_any_beam_set(n, cell, f, f_y, alpha, M, px, py, step):
+    sim = plan(n, cell, f, 21, f_y=f_y, alpha=alpha)
+    assert max(sim.beams()[0]) == M
+    x, y = np.meshgrid(step * np.arange(px) - 1.3, step * np.arange(py) - 0.7)
+    pos = (x.ravel(), y.ravel())
+    out = scan(sim, pos, px, py, P.PRISM_SCAN_ROWS)
+    some = np.array([0, px - 1, px * py // 2, px * py - 1])
+    close(out[some], exact(sim, cell, f, f_y, pos[0][some], pos[1][some]), sim.info.n_beams)
+    sim.close()
+
+
+@pytest.mark.parametrize("n,cell,f", [(64, 8.0, 2), (256, 16.0, 4), (256, 12.5, 2)])
+def test_small_value_and_remainder_rasters_by_rows(n, cell, f):
+    sim = plan(n, cell, f, 22, precision=P.PRISM_PRECISION_FP16X2)
+    x, y = np.meshgrid(0.3 * np.arange(4) - 0.5, 0.3 * np.arange(4) - 0.5)
+    pos = (x.ravel(), y.ravel())
+    out = scan(sim, pos, 4, 4, P.PRISM_SCAN_ROWS)
+    ref = exact(sim, cell, f, 0, *pos)
+    beams = sim.info.n_beams
+    assert np.linalg.norm(out - ref) / np.linalg.norm(ref) <= 2.0 * (2.0 ** -20 * beams ** 0.5 + (beams + 24) * 2.0 ** -24)
+    sim.close()
