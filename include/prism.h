@@ -27,7 +27,15 @@
  *   - Determinism: the same inputs give bitwise-identical outputs (fixed reduction trees; the
  *     only atomics hand out work units -- column tiles, probe blocks -- and which CTA
  *     computes a unit changes no result), autotuned or not; only a plan tuned with the FFT radix
- *     variants (PRISM_AUTOTUNE_FFT_RADIX) may pick another rounding by timing.
+ *     variants (PRISM_AUTOTUNE_FFT_RADIX) may pick another rounding by timing.  A scan takes one of
+ *     several paths (prism_plan_scan_path) by the raster's sides and positions, and, for rasters that
+ *     go by rows, by the memory for their scratch: a plan's or batch's HBM budget, and device memory
+ *     itself, may send such a raster another way.  The paths agree to FP32 rounding (16-bit and
+ *     value + remainder storage: to that of their coefficients), not bit for bit, so a probe's result
+ *     may differ in rounding between a raster and a part of it, or between a batch or a server under
+ *     a budget and a plan without one.  On one path it does not depend on the other probes: bands of
+ *     whole raster rows that all go by rows, and parts that all go by blocks, equal the whole bit for
+ *     bit.
  *   - A plan's calls run on its stream, one after another: its scratch and its work-unit
  *     counters are the plan's, so calls on one plan must not overlap (different plans may).
  *   - Memory: the caller owns every pointer it passes in; the plan owns the transmission
@@ -76,7 +84,8 @@ extern "C" {
  *                FP16 value plus the FP16 rounding of its remainder and three tensor-core products
  *                per step (value x value + value x remainder + remainder x value), FP32-class
  *                accuracy with the storage of FP32. (Rasters whose rows of 3 or more probes each share
- *                one y are summed by rows in FP32 from the unpacked values instead.)  The build
+ *                one y are summed by rows in FP32 from the unpacked values instead, where that pays
+ *                and the scratch for it fits.)  The build
  *                (transmission, FFTs, propagator) is FP32 in every mode.  Ignored by
  *                multislice_scan_run.  Zero-initialised structs select FP32.
  *   f_y          interpolation factor along y when it differs from f (f is then the factor along
@@ -207,8 +216,9 @@ int prism_scan_run_accumulate(prism_plan *plan, const prism_probe *probe, const 
  * sum |Psi0|^2, annular bins.  Same grid rules as a plan (f, downsample and alpha_max are
  * ignored).  V_dev as above, out_dev float32 [py][px][nbins].  Uses its own stream-ordered
  * scratch on `cuda_stream`, sized to at most max(1, scratch_bytes / (8 nx ny)) probes in flight
- * (scratch_bytes = 0: 1 GiB).  Asynchronous; synchronise the stream before reading out_dev.  From
- * 256^2 to 1024^2 the column passes stage their tiles through TMA with bounded waits; a wait that runs out
+ * (scratch_bytes = 0: 1 GiB).  Asynchronous; synchronise the stream before reading out_dev.  At
+ * n_y = 1024, and at 512 and 256 from some 8000 and 16 000 kept columns of all probes in flight on, the
+ * column passes stage their tiles through TMA with bounded waits; a wait that runs out
  * (which would leave a wave incomplete) makes that batch's bins NaN. */
 int multislice_scan_run(const prism_grid *grid, const float *V_dev, const prism_probe *probe,
                         const prism_scan *scan, const prism_detector *det, float *out_dev,
@@ -287,8 +297,10 @@ typedef struct prism_server prism_server;
  * (its S-matrix plan unless resident, output and positions) fits hbm_budget_bytes (0 = no
  * budget), evicting idle resident S-matrices least-recently-used when needed; a request that does
  * not fit yet does not hold back later ones.  Requests on different S-matrices run on different
- * streams and overlap on the device.  Results equal those of the request run alone (the kernels
- * are deterministic).  (No counterpart in the paper: this is the serving form of the method.) */
+ * streams and overlap on the device.  Results equal those of the request run alone on a server with
+ * or without a budget as this one (the kernels are deterministic), to rounding where the device had no memory
+ * left for a scan's scratch (Determinism, above).  (No counterpart in the paper: this is the
+ * serving form of the method.) */
 int prism_server_create(size_t hbm_budget_bytes, int max_inflight, prism_server **out);
 /* Queue a request; returns a ticket.  Errors: INVALID for malformed requests. */
 int prism_server_submit(prism_server *server, const prism_request *req, unsigned long long *ticket);
@@ -325,9 +337,8 @@ void prism_server_destroy(prism_server *server);
  * S-matrix is untouched).  The paper has no counterpart. */
 #define PRISM_TUNE_ROW 0
 #define PRISM_TUNE_COL 1
-#define PRISM_TUNE_SCAN 2  /* contraction tile shape of the FP32 GEMM scan (prism_plan_autotune_scan); a raster
-                              whose rows of 3 or more probes each share one y goes by rows, and positions too
-                              far apart to share S values probe by probe, for which every shape is the same */
+#define PRISM_TUNE_SCAN 2  /* contraction tile shape of the FP32 GEMM scan (prism_plan_autotune_scan); scans that
+                              go by rows or probe by probe (prism_plan_scan_path) are the same for every shape */
 #define PRISM_TUNE_SCAN_TC 3  /* ring shape of the tensor-core scan of a 16-bit plan: stages x K values of
                                  its A operand (3 x 96 default, 2 x 128, 4 x 64; split mode 2 x 32 only) */
 #define PRISM_TUNE_MAX_SHAPES 16

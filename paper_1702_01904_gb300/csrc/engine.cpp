@@ -1018,8 +1018,8 @@ static size_t block_scratch(const prism_plan *P, int px, int py) {
 // distinct m and window pixel; in blocks (scan_gemm.cuh, scan_tc.cuh) each probe costs one per beam and
 // window pixel.  Measured over windows of 32 to 128 pixels, 49 to 529 beams, steps of 0.1 to 2 A and
 // rasters of 2 x 2 to 64 x 64: 1.2 to 6.6 times the speed of the FP32 blocks wherever the test below lets
-// rows of 3 or more through, 0.84 to 1.06 times for tall rasters of rows of 2.  The 16-bit precisions round
-// the coefficients of every beam and probe, which do not separate: they stay with the tensor cores.
+// rows of 3 or more through, 0.84 to 1.06 times for tall rasters of rows of 2.  FP16 and BF16 S-matrices stay
+// with the tensor cores, whose products take 16-bit coefficients.
 // Sets a.rows_lp > 0, the columns and the rows held at once, or leaves a.rows_lp = 0.
 static void raster_rows(const prism_plan *P, const prism_scan *sc, const ScanExtent &ext, ScanArgs &a) {
     const bool split = P->prec == PRISM_PRECISION_FP16X2;
@@ -1285,10 +1285,6 @@ static int split_counters(prism_plan *P, ScanArgs &a, int grid) {
     return PRISM_OK;
 }
 
-// FP32 mode: the CUDA-core scan kernels; 16-bit mode: the tensor-core kernel (persistent grid, its
-// window scratch grown on demand)
-// FP32: the raster-row scan where it applies (raster_rows), the GEMM scan over 8 x 4 raster blocks when its shared memory fits (grid > 0), else the
-// grouped / per-probe kernels (grid 0); 16-bit: the tensor-core scan
 // the GEMM scan's contraction shape in use: the tuned or pinned one where it is compiled for the
 // plan's window, else the default
 static int gemm_shape(const prism_plan *P) {
@@ -1300,7 +1296,10 @@ static int tc_shape(const prism_plan *P) {
     return P->tc_shape > 0 && P->tc_shape < scan_tc_shapes(tc_mode(P->prec)) ? P->tc_shape : 0;
 }
 
-// The grid and the bytes of scratch (and of counters) of the path a scan takes; grid 0: kernels that need none
+// The grid and the bytes of scratch (and of counters) of the path a scan takes.  FP32: by raster rows or probe by
+// probe where those apply (raster_rows, position_list), else the GEMM scan over 4 x 8 raster blocks when its
+// shared memory fits, else the grouped / per-probe kernels (grid 0).  16-bit: by rows, or the tensor-core scan
+// (persistent grids, their window scratch grown on demand).
 static int scan_scratch(const prism_plan *P, const ScanArgs &a, int *grid, size_t *win, size_t *cnt) {
     *grid = 1;
     *win = *cnt = 0;

@@ -99,7 +99,10 @@ static int tune_row_find(int thr, bool stg, bool tma) {
 // unstaged).  N = 512: 384 threads staged by cp.async from 16 384 rows on (213 beams: 123 us against
 // 132 for 128 threads unstaged; 829 beams 446 against 490; 49 beams 33.4 against 33.5; with 13 beams,
 // 6656 rows, the small CTAs are faster, 12.9 against 14.0).  In a batch graph, whose branches share the
-// SMs, the default launcher's smaller CTAs (the 1024 shape holds 163 KB of shared memory per CTA).
+// SMs, the default launcher: smaller CTAs up to N = 1024 (the 1024 shape holds 163 KB of shared memory per CTA).
+// At N = 2048 it is one CTA of 384 threads per SM there too, which loses less by the other branches' kernels than
+// it gains: four 2048^2 cells in 4 branches 51.4 ms per run, with CTAs of 128 threads 55.8; two beside six
+// 1024^2 cells 31.2 against 32.9; one beside twelve 256^2 cells 14.1 against 14.4.
 int tune_row_default(int nx, long long rows, bool shared) {
     if (shared) return -1;
     const int v = nx == 1024 ? tune_row_find(384, false, true) : nx == 512 && rows >= 16384 ? tune_row_find(384, true, false) : -1;

@@ -91,8 +91,9 @@ struct RowCfg {
     static constexpr int EXI = FS::N2 * (FS::N1 + 1);
     static constexpr int EX = EXF > EXI ? EXF : EXI;
     static constexpr int SLOT_F2 = (TMA ? NX / 2 : STAGE ? NX : 0) + EX;  // staging row + exchange, float2
-    // at N = 2048 the two stage-twiddle tables (32 KB) would hold the CTAs to 2 per SM: there they are
-    // read through L1 (read-only path), interleaved with the exchange stores, for 3 CTAs per SM
+    // at N = 2048 the two stage-twiddle tables (32 KB) would hold the warps to 8 per SM: there they are
+    // read through L1 (read-only path), interleaved with the exchange stores, for 12 (one CTA of 384 threads,
+    // the default, or three of 128)
     static constexpr bool L1TW = NX >= 2048;
     static constexpr bool LOCKSTEP = NX >= 2048 && THR >= 384;
     static constexpr int TW_MODE = L1TW ? TW_GLOBAL : TW_SMEM;

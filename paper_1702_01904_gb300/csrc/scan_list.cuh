@@ -3,9 +3,9 @@
 // several beams' loads in flight; the window then goes through shared memory for its transform and bins.
 //
 // Bound by the S values read, B nw^2 8 bytes per probe once from the L2 (900 scattered probes of 129 beams
-// and 64-pixel windows: 3.8 GB in 0.34 ms).  The blocks of scan_gemm.cuh run such probes one after another
+// and 64-pixel windows: 3.8 GB in 0.33 ms).  The blocks of scan_gemm.cuh run such probes one after another
 // with one warp in eight at work, and a list of positions fills 4 of their 32 slots: 1.32 ms for those 900,
-// 0.32 for 10 of them (35 us here).  900 jittered positions of 32 x 16 windows and 25 beams: 69 -> 20 us on
+// 0.32 for 10 of them (29 us here).  900 jittered positions of 32 x 16 windows and 25 beams: 69 -> 20 us on
 // the device.
 // Few probes: a cluster of up to 8 CTAs shares a probe's beams, and their windows are added in the first
 // one's shared memory, rank by rank.  Bins of short lists (up to 1024-pixel windows) take a thread each

@@ -8,8 +8,10 @@
 // different streams and overlap on the device; requests that share a key reuse the resident
 // S-matrix (the S-matrix serves every later probe configuration, Varying Probe Size section).
 // Idle resident S-matrices are evicted least-recently-used when a new one needs the memory.
-// Every wait is bounded.  Results are bitwise identical to running the request alone: the
-// kernels are deterministic and nothing is shared between in-flight requests but read-only S.
+// Every wait is bounded.  Results are bitwise identical to running the request alone on a server with or
+// without a budget as this one: the kernels are deterministic and nothing is shared between in-flight
+// requests but read-only S (where the device has no memory left for the scratch of a raster that goes by
+// rows, it goes another way, the same to rounding).
 #include <cuda_runtime.h>
 
 #include <algorithm>
