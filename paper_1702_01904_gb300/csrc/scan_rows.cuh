@@ -23,8 +23,8 @@
 // 2048^2 cell (529 beams, 128-pixel windows) 2.70 -> 0.73 ms; 16 x 16 probes of a 256^2 cell 68 -> 25 us.
 // 33 x 31 probes of a 512^2 cell from value + remainder storage (213 beams): 382 us on the tensor cores,
 // 110 us here, nearer to 64 bits (2.3e-6 against 4.9e-6 off).
-// Bound: k_rows_sum by the load/store pipe (67 % busy; its S reads hit the L2, 1.9 GB of them),
-// k_rows_window by the same pipe (60 %) and dependent latency at 16 warps per SM (issue slots 49 %);
+// Bound: k_rows_sum by the load/store pipe (57 % busy) and its loads' latency at 16 warps per SM (its S reads hit
+// the L2, 1.9 GB of them), k_rows_window by the same pipe (61 %) and dependent latency (issue slots 49 %);
 // leaving out the products saves 32 % of its time, the loads of the planes 20 %, the transforms 12 %,
 // the bins 8 %, the folding 5 %.
 // Against 64 bits from the same S (10 grids, windows of 16 to 128 pixels, 13 to 529 beams): 3 wide bins 0.28 to
