@@ -1053,11 +1053,12 @@ static void raster_rows(const prism_plan *P, const prism_scan *sc, const ScanExt
     // Where no HBM budget is given, at least 128 MB: a tall raster of few columns has few blocks, and the rows
     // that their scratch held went launch by launch (value + remainder storage, 4 x 99 probes of 49 beams and
     // 32-pixel windows: 56 us on the tensor cores, 1031 us one row at a time; 3 x 75 of 213 beams and
-    // 64-pixel windows: 132, 334).  Under a batch's tight budget no more than the blocks would take of
-    // this very scan.
-    if (P->scratch_budget) most = std::min(most, block_scratch(P, sc->px, sc->py));
-    else if (!P->budget) most = std::max<size_t>(most, (size_t)128 << 20);
+    // 64-pixel windows: 132, 334).  Not for 64 MB of unpacked values and more: 32 x 32 probes 2 A apart reach
+    // 103 MB of S, whose unpacking costs more than the rows save (144 us on the tensor cores, 160).  Under a
+    // batch's tight budget no more than the blocks would take of this very scan.
     const size_t unpacked = split ? (size_t)P->nbeams * rows * cols * sizeof(float2) : 0;
+    if (P->scratch_budget) most = std::min(most, block_scratch(P, sc->px, sc->py));
+    else if (!P->budget && unpacked < (size_t)64 << 20) most = std::max<size_t>(most, (size_t)128 << 20);
     if (unpacked + row > most) return;
     const size_t limit = std::min<size_t>(most - unpacked, (size_t)384 << 20);
     size_t chunk = std::min<size_t>(limit / row, sc->py);

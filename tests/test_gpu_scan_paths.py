@@ -480,3 +480,11 @@ def test_small_value_and_remainder_rasters_by_rows(n, cell, f):
     beams = sim.info.n_beams
     assert np.linalg.norm(out - ref) / np.linalg.norm(ref) <= 2.0 * (2.0 ** -20 * beams ** 0.5 + (beams + 24) * 2.0 ** -24)
     sim.close()
+
+
+def test_wide_value_and_remainder_rasters_are_not_unpacked():
+    # 32 x 32 probes 2 A apart reach the whole S-matrix (103 MB unpacked) for few windows on any part of it
+    sim = plan(1024, 64.0, 16, 23, precision=P.PRISM_PRECISION_FP16X2)
+    x, y = np.meshgrid(2.0 * np.arange(32), 2.0 * np.arange(32))
+    scan(sim, (x.ravel(), y.ravel()), 32, 32, P.PRISM_SCAN_TENSOR)
+    sim.close()
