@@ -488,3 +488,21 @@ def test_wide_value_and_remainder_rasters_are_not_unpacked():
     x, y = np.meshgrid(2.0 * np.arange(32), 2.0 * np.arange(32))
     scan(sim, (x.ravel(), y.ravel()), 32, 32, P.PRISM_SCAN_TENSOR)
     sim.close()
+
+
+def test_parts_of_a_raster_agree_to_rounding():
+    # a raster by rows against its bands of 6 rows (24 probes: a list), of whole rows that go by rows (bit for bit),
+    # and its two left columns
+    sim = plan(256, 16.0, 4, 24)
+    beams = sim.info.n_beams
+    x, y = np.meshgrid(0.2 * np.arange(4), 0.2 * np.arange(24))
+    whole = scan(sim, (x.ravel(), y.ravel()), 4, 24, P.PRISM_SCAN_ROWS)
+    for r in range(0, 24, 6):
+        band = scan(sim, (x[r:r + 6].ravel(), y[r:r + 6].ravel()), 4, 6, P.PRISM_SCAN_LIST)
+        close(band, whole[4 * r:4 * (r + 6)].astype(np.float64), beams)
+    for r in range(0, 24, 8):
+        band = scan(sim, (x[r:r + 8].ravel(), y[r:r + 8].ravel()), 4, 8, P.PRISM_SCAN_ROWS)
+        assert np.array_equal(band, whole[4 * r:4 * (r + 8)])
+    left = scan(sim, (x[:, :2].ravel(), y[:, :2].ravel()), 2, 24, P.PRISM_SCAN_LIST)
+    close(left, whole.reshape(24, 4, -1)[:, :2].reshape(48, -1).astype(np.float64), beams)
+    sim.close()
